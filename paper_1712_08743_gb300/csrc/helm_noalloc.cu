@@ -82,10 +82,9 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
         slot[b] = k;
     }
     // the coarse end of the cycle helm_vcycle would use: the dense inverse of level m->ld where it
-    // applies (beta2 != 0 and the inversion fits the GPU), else the shared-memory tail
-    int W = 0, per = 0;
+    // applies (beta2 != 0), else the shared-memory tail
     const bool dense = nrhs <= kDenseAutoMaxRhs && beta2 != 0.0 && m->ld > 0 &&
-                       dense_invert_plan((int)m->lv[m->ld].n(), false, &W, &per);
+                       dense_invert_fits(m->lv[m->ld].nx, m->lv[m->ld].nz);
     // groups of consecutive right-hand sides sharing a slot, at most 8 each
     int grp[kNoAllocMaxRhs + 1];
     int ngroups = 0, maxg = 0;
@@ -107,7 +106,7 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
     const size_t o_grp = take(sizeof(int) * (ngroups + 1));
     const size_t common = off;
     struct Plan {
-        size_t minv = 0, work = 0, md = 0, panel = 0, dinv = 0, bar = 0, err = 0, fbar = 0, ferr = 0;
+        size_t minv = 0, work = 0, md = 0, err = 0, fbar = 0, ferr = 0;
         size_t f[kMaxLevels] = {}, e[kMaxLevels] = {}, g[kMaxLevels] = {};
         int top = 0;
         size_t end = 0;
@@ -117,11 +116,7 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
         off = common;
         if (dn) {
             const size_t nd = m->lv[m->ld].n();
-            const int nl = std::min(per, nslots);
             p.minv = take(sizeof(float2) * nd * nd * nslots);
-            p.panel = take(sizeof(float2) * 2 * nd * W * nl);
-            p.dinv = take(sizeof(float2) * 2 * (size_t)W * W * nl);
-            p.bar = take(sizeof(unsigned) * nl);
             p.err = take(sizeof(int));
             p.fbar = take(sizeof(unsigned));   // the persistent F-cycle's barrier and error flag
             p.ferr = take(sizeof(int));
@@ -162,14 +157,11 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_grp, grp, sizeof(int) * (ngroups + 1), cudaMemcpyHostToDevice, s);
     bool use_dense = dense;
     if (e == cudaSuccess && use_dense) {
-        // every byte the inversion reads is written earlier in this call (the counters and the
-        // error flag are cleared by the launcher), so stale contents do not matter
+        // every byte the inversion reads is written earlier in this call (the error flag is
+        // cleared by the launcher), so stale contents do not matter
         e = launch_dense_invert<float>(level_dev(m, m->ld, true), reinterpret_cast<const double*>(base + o_w2s),
-                                       reinterpret_cast<const int*>(base + o_mods), nslots, beta1, beta2, W, per,
+                                       reinterpret_cast<const int*>(base + o_mods), nslots, beta1, beta2,
                                        reinterpret_cast<float*>(base + plan.minv),
-                                       reinterpret_cast<float*>(base + plan.panel),
-                                       reinterpret_cast<float*>(base + plan.dinv),
-                                       reinterpret_cast<unsigned*>(base + plan.bar),
                                        reinterpret_cast<int*>(base + plan.err), s);
         int herr = -1;
         if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, base + plan.err, sizeof(int), cudaMemcpyDeviceToHost, s);

@@ -681,7 +681,7 @@ static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* r
 // copies). One inverse per distinct (model, frequency) pair: slot[b].
 struct CoarseSet {
     DBuf work, mf, md, slot, w2s, mods;
-    DBuf grp, panel, dinv, bar, err;   // dense path
+    DBuf grp, err;                     // dense path
     int n = 0, nslots = 0;
     int ld = 0;                        // > 0: the dense path, level ld
     int ngroups = 0, maxg = 0;
@@ -717,13 +717,11 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
     HELM_CUDA_TRY(cudaMemcpyAsync(cs.w2s.p, w2s.data(), sizeof(double) * cs.nslots, cudaMemcpyHostToDevice, s));
     HELM_CUDA_TRY(cudaMemcpyAsync(cs.mods.p, mods.data(), sizeof(int) * cs.nslots, cudaMemcpyHostToDevice, s));
 
-    int W = 0, per = 0;
     const bool want_dense = coarse == HELM_COARSE_DENSE || coarse == HELM_COARSE_FUSED ||
                             (coarse == HELM_COARSE_AUTO && nrhs <= kDenseAutoMaxRhs);
-    if (want_dense && b2 != 0.0 && m->ld > 0 && dense_invert_plan((int)m->lv[m->ld].n(), dbl, &W, &per)) {
+    if (want_dense && b2 != 0.0 && m->ld > 0 && dense_invert_fits(m->lv[m->ld].nx, m->lv[m->ld].nz)) {
         const int ld = m->ld, n = (int)m->lv[ld].n();
         const size_t es = dbl ? sizeof(double2) : sizeof(float2);
-        const int nl = std::min(per, cs.nslots);
         // groups of at most kDenseGroup consecutive right-hand sides of one slot
         std::vector<int> grp{0};
         int maxg = 0;
@@ -734,19 +732,14 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
             }
         DBuf& mi = dbl ? cs.md : cs.mf;
         TRY_ALLOC(mi, es * (size_t)n * n * cs.nslots, s);
-        TRY_ALLOC(cs.panel, es * 2 * (size_t)n * W * nl, s);
-        TRY_ALLOC(cs.dinv, es * 2 * (size_t)W * W * nl, s);
-        TRY_ALLOC(cs.bar, sizeof(unsigned) * nl, s);
         TRY_ALLOC(cs.err, sizeof(int), s);
         TRY_ALLOC(cs.grp, sizeof(int) * grp.size(), s);
         HELM_CUDA_TRY(cudaMemcpyAsync(cs.grp.p, grp.data(), sizeof(int) * grp.size(), cudaMemcpyHostToDevice, s));
         const LevelDev Ld = level_dev(m, ld, true);
-        cudaError_t e = dbl ? launch_dense_invert<double>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1, b2, W,
-                                                          per, cs.md.as<double>(), cs.panel.as<double>(),
-                                                          cs.dinv.as<double>(), cs.bar.as<unsigned>(), cs.err.as<int>(), s)
-                            : launch_dense_invert<float>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1, b2, W,
-                                                         per, cs.mf.as<float>(), cs.panel.as<float>(),
-                                                         cs.dinv.as<float>(), cs.bar.as<unsigned>(), cs.err.as<int>(), s);
+        cudaError_t e = dbl ? launch_dense_invert<double>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1,
+                                                          b2, cs.md.as<double>(), cs.err.as<int>(), s)
+                            : launch_dense_invert<float>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1,
+                                                         b2, cs.mf.as<float>(), cs.err.as<int>(), s);
         int herr = -1;
         if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, cs.err.p, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -757,7 +750,7 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
             cs.maxg = maxg;
             return HELM_OK;
         }
-        // the dense inverse could not be formed (a launch that does not fit, or a
+        // the dense inverse could not be formed (a failed launch, or a
         // vanishing pivot): fall back to the multigrid tail below
         cudaGetLastError();
     }
