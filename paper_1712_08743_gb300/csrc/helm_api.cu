@@ -95,6 +95,18 @@ int create_model(helm_ctx* ctx, cudaStream_t s, int Px, int Pz, double h, const 
         return HELM_E_INVALID;
     }
     const int L = (int)m->lv.size() - 1;
+    // P^T G P of a constant symmetric stencil (centre c, edge e, corner a) with the bilinear P:
+    // sums of dyadic fractions, so exactly what the device forms node by node. The corner
+    // couples corner supports, the edge sums over a shared side (the 5-point stencil is c = 4,
+    // e = -1, a = 0; the fixed point 8/3, -1/3, -1/3 is the bilinear element's).
+    for (double c = 4.0, e = -1.0, a = 0.0, l = 1; l <= L; ++l) {
+        const double c2 = 2.25 * c + 6.0 * e + 4.0 * a;
+        const double e2 = 0.375 * c + 2.0 * e + 2.0 * a;
+        const double a2 = 0.0625 * c + 0.5 * e + 1.0 * a;
+        c = c2; e = e2; a = a2;
+        double* g = m->lv[(size_t)l].g0;
+        g[0] = c; g[1] = e; g[2] = a;
+    }
     m->lf = L;
     for (int l = 1; l <= L; ++l)
         if (m->lv[l].n() <= (size_t)kFcycleMaxPoints) { m->lf = l; break; }

@@ -55,6 +55,8 @@ struct LevelDev {
     size_t mstride;
     const void* gk;     // Galerkin levels: float* or double* [nmodels][10][n]
     size_t gkstride;
+    int gconst;         // Galerkin levels: 1 where G is the stencil g0 at every node off the border
+    float g0[3];        // (constant density): centre, east = north, north-east = north-west
     const void* rho;    // finest level with a density (Eq. 1): [3][n] east-edge, north-edge and diagonal
                         // coefficients of the flux-form operator; nullptr for constant density
 };
@@ -68,6 +70,7 @@ struct Level {
     double* gkd = nullptr;
     float* rhof = nullptr;   // finest level with a density: [3][n] (see LevelDev::rho)
     double* rhod = nullptr;
+    double g0[3] = {0, 0, 0};   // G of a Galerkin level off the border (constant density)
     size_t n() const { return (size_t)nx * nz; }
 };
 
@@ -186,6 +189,8 @@ inline LevelDev level_dev(const helm_model* m, int l, bool dbl) {
     d.mstride = m->nmodels > 1 ? L.n() : 0;
     d.gk = dbl ? (const void*)L.gkd : (const void*)L.gkf;
     d.gkstride = m->nmodels > 1 ? kGalerkinCoefs * L.n() : 0;
+    d.gconst = !m->vd && l > 0;
+    for (int k = 0; k < 3; ++k) d.g0[k] = (float)L.g0[k];
     d.rho = dbl ? (const void*)L.rhod : (const void*)L.rhof;
     return d;
 }
@@ -272,6 +277,16 @@ void launch_correct_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2
 template <typename T>
 void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double b1, double b2,
                      double wj, const T* f, T* fc, const RhsState* st, int nrhs, cudaStream_t s, int tile = 1);
+// The same steps for batches above kGalMarchMinRhs, complex64 (helm_gal_march.cu): smaller
+// batches leave most warps of the march without a right-hand side, and the tiles' shorter
+// chains are what counts there.
+constexpr int kGalMarchMinRhs = 16;
+void launch_gal_march_restrict(bool correct, const LevelDev& Lf, const LevelDev& Lc, const float* hw, double b1,
+                               double b2, double wj, const float* f, const float* ec, float* fc, const RhsState* st,
+                               int nrhs, cudaStream_t s);
+void launch_gal_march_prolong(const LevelDev& Lf, const LevelDev& Lc, const float* hw, double b1, double b2,
+                              double wj, const float* f, const float* ec, float* out, const RhsState* st, int nrhs,
+                              cudaStream_t s, int accumulate);
 // The prolongation of Galerkin level l + 1 (from e of level l + 2; right-hand side
 // fm, added to em when acc_m) and then that of level l (right-hand side fl, into
 // out, added to it when acc_f), in one launch; level l + 1's correction stays in
