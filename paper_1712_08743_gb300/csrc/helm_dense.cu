@@ -83,18 +83,31 @@ constexpr int kTriMaxW = 36;      // shared tiles of the widest instance (48 KB 
 constexpr int kTriThreads = 256;  // 16 x 16, each thread RT x RT elements of the w x w matrix
 constexpr int kTriCols = 8;       // columns of a block column per block of k_dense_columns
 
-// 1 / d of a pivot block, d = |det|^2. Float: one Newton step x + x (1 - d x) on the
-// approximate reciprocal, with no IEEE divide behind a branch (either its test or its call
-// costs every step: 284 against 226 us for the 1024-node level); d outside pivot_ok's
-// range is reported like a vanishing pivot. Double: the divide (Newton steps from a float
-// seed measured the same).
-__device__ __forceinline__ float pivot_rcp(float d) {
-    const float x = __fdividef(1.0f, d);
-    return fmaf(x, fmaf(-d, x, 1.0f), x);
+// 1 / det of a pivot block; false if it vanishes or is not finite. Float: |det|^2 inverted by one
+// Newton step x + x (1 - d x) on the approximate reciprocal; an IEEE divide behind its range
+// test costs every step (284 against 226 us for the 1024-node level), and so does scaling each
+// determinant (271 us). The range left, |det| within 1e-18 .. 3e18, is that of pivots within nine
+// decimal orders of 1, and the matrix is scaled for it (tri_scale). Double: the divide (Newton
+// steps from a float seed measured the same).
+__device__ __forceinline__ bool pivot_inv(cx<float> det, cx<float>& inv) {
+    const float d = det.re * det.re + det.im * det.im;
+    float x = __fdividef(1.0f, d);
+    x = fmaf(x, fmaf(-d, x, 1.0f), x);
+    inv = cx<float>(det.re * x, -det.im * x);
+    return d > 1e-37f && d < 1e37f;
 }
-__device__ __forceinline__ double pivot_rcp(double d) { return 1.0 / d; }
-__device__ __forceinline__ bool pivot_ok(float d) { return d > 1e-37f && d < 1e37f; }
-__device__ __forceinline__ bool pivot_ok(double d) { return d > 0.0 && isfinite(d); }
+__device__ __forceinline__ bool pivot_inv(cx<double> det, cx<double>& inv) {
+    const double d = det.re * det.re + det.im * det.im, id = 1.0 / d;
+    inv = cx<double>(det.re * id, -det.im * id);
+    return d > 0.0 && isfinite(d);
+}
+// The power of two that brings the level's first diagonal entry near 1: the matrix is inverted
+// scaled by it (exactly), so the frequency's magnitude does not eat the pivots' range.
+__device__ __forceinline__ double tri_scale(const double* __restrict__ gk, size_t n, double hb1, double hb2) {
+    const double g = __ldg(gk), q = __ldg(gk + 5 * n);
+    const double v = fmax(fabs(g - hb1 * q), fabs(hb2 * q));
+    return v > 0.0 && isfinite(v) ? exp2(-(double)ilogb(v)) : 1.0;
+}
 
 // In-place Gauss-Jordan inversion of a w x w matrix by 2 x 2 pivot blocks without pivoting
 // (see the head of this file; half the barriers of single pivots): thread (ti, tj) =
@@ -126,10 +139,8 @@ __device__ __forceinline__ bool gj_invert(cx<T> (&a)[RT][RT], int w, int ti, int
                 };
                 const cx<T> p00 = from(kk), p01 = from(kk + 1), p10 = from(16 + kk), p11 = from(17 + kk);
                 const cx<T> det = p00 * p11 - p01 * p10;
-                const T d = det.re * det.re + det.im * det.im;
-                ok = ok && pivot_ok(d);
-                const T id = pivot_rcp(d);
-                const cx<T> di(det.re * id, -det.im * id);
+                cx<T> di;
+                ok = pivot_inv(det, di) && ok;
                 // this half-warp's row of the inverse: row 0 is (p11, -p01) / det, row 1 (-p10, p00) / det
                 const cx<T> q0 = half ? cx<T>(-p10.re, -p10.im) : p11, q1 = half ? p00 : cx<T>(-p01.re, -p01.im);
                 const cx<T> i0 = di * q0, i1 = di * q1;
@@ -191,7 +202,8 @@ __global__ void __launch_bounds__(kTriThreads) k_dense_chain(TriShape sh, const 
     const double hw = w2s[blockIdx.y], hb1 = hw * b1, hb2 = hw * b2;
     const double* gk = gkall + (size_t)mods[blockIdx.y] * gkstride;
     T* out = minv + 2 * (size_t)n * n * blockIdx.y;
-    auto form = [&](double2 e) { return cx<T>((T)(e.x - hb1 * e.y), (T)(hb2 * e.y)); };
+    const double sc = tri_scale(gk, (size_t)n, hb1, hb2);
+    auto form = [&](double2 e) { return cx<T>((T)(sc * (e.x - hb1 * e.y)), (T)(sc * (hb2 * e.y))); };
     auto raw = [&](int kr, int r, int kc, int q) -> double2 {
         if (r < 0 || r >= w) return make_double2(0.0, 0.0);
         return gal_raw(gk, (size_t)n, sh.nx, sh.node(kr, r), sh.node(kc, q));
@@ -293,6 +305,7 @@ __global__ void __launch_bounds__(kTriThreads) k_dense_columns(TriShape sh, cons
     const int j = nb - 1 - blockIdx.x, c0 = blockIdx.y * kTriCols, cw = min(kTriCols, w - c0);
     const double hw = w2s[blockIdx.z];
     const double* gk = gkall + (size_t)mods[blockIdx.z] * gkstride;
+    const double sc = tri_scale(gk, (size_t)n, hw * b1, hw * b2);
     T* out = minv + 2 * (size_t)n * n * blockIdx.z;
     const int2 bd = j > 0 ? sh.scratch((nb - 1) + j - 1) : make_int2(0, 0);
     const int2 bu = j < nb - 1 ? sh.scratch(2 * (nb - 1) + j) : make_int2(0, 0);
@@ -308,7 +321,7 @@ __global__ void __launch_bounds__(kTriThreads) k_dense_columns(TriShape sh, cons
                 if (j < nb - 1) v = v + ldcc(out, sh.at(bu, p, q));
                 if (j > 0 && j < nb - 1 && p - q <= 1 && q - p <= 1) {
                     const double2 e = gal_raw(gk, (size_t)n, sh.nx, sh.node(j, p), sh.node(j, q));
-                    v = v - cx<T>((T)(e.x - hw * b1 * e.y), (T)(hw * b2 * e.y));
+                    v = v - cx<T>((T)(sc * (e.x - hw * b1 * e.y)), (T)(sc * (hw * b2 * e.y)));
                 }
             }
             a[r][c] = v;
@@ -327,6 +340,7 @@ __global__ void __launch_bounds__(kTriThreads) k_dense_columns(TriShape sh, cons
     for (int r = 0; r < RT; ++r)
 #pragma unroll
         for (int c = 0; c < RT; ++c) {
+            a[r][c] = (T)sc * a[r][c];   // the inverse of the unscaled matrix
             const int p = ti + 16 * r, q = tj + 16 * c - c0;
             if (p < w && q >= 0 && q < kTriCols) {
                 Y[0][p][q] = a[r][c];
