@@ -12,11 +12,6 @@ using namespace helm;
 
 namespace {
 
-struct DevMem {   // synchronous device allocation for API-level staging
-    void* p = nullptr;
-    ~DevMem() { if (p) cudaFree(p); }
-};
-
 class DeviceGuard {   // makes the context's device current for the call
   public:
     explicit DeviceGuard(int dev) {
@@ -54,6 +49,7 @@ int check_opts(const helm_solve_opts& o) {
 
 struct helm_fwi_state {
     helm_model* m = nullptr;
+    int device = 0;
     helm::FwiState* st = nullptr;
 };
 
@@ -128,34 +124,46 @@ int create_model(helm_ctx* ctx, cudaStream_t s, int Px, int Pz, double h, const 
         helm_destroy_model(m);
         return e == cudaErrorMemoryAllocation ? HELM_E_NOMEM : HELM_E_CUDA;
     };
-    cudaError_t e = cudaMalloc(&m->m_pad, sizeof(double) * m->n() * nmodels);
-    if (e != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc(&m->lv[0].m2f, sizeof(float) * m->n() * nmodels)) != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc(&m->lv[0].m2d, sizeof(double) * m->n() * nmodels)) != cudaSuccess) return fail(e);
-    if (m->vd) {
-        Level& L0 = m->lv[0];
-        if ((e = cudaMalloc(&L0.rhof, sizeof(float) * 3 * L0.n())) != cudaSuccess) return fail(e);
-        if ((e = cudaMalloc(&L0.rhod, sizeof(double) * 3 * L0.n())) != cudaSuccess) return fail(e);
-        if ((e = cudaMalloc(&L0.gkf, sizeof(float) * kGalerkinCoefs * L0.n())) != cudaSuccess) return fail(e);
-        if ((e = cudaMalloc(&L0.gkd, sizeof(double) * kGalerkinCoefs * L0.n())) != cudaSuccess) return fail(e);
-    }
-    for (int l = 1; l <= L; ++l) {
-        Level& Lv = m->lv[l];
-        if ((e = cudaMalloc(&Lv.gkf, sizeof(float) * kGalerkinCoefs * Lv.n() * nmodels)) != cudaSuccess) return fail(e);
-        if ((e = cudaMalloc(&Lv.gkd, sizeof(double) * kGalerkinCoefs * Lv.n() * nmodels)) != cudaSuccess) return fail(e);
-    }
     std::vector<int> opsf[2], opsv[2];
     for (int d = 0; d < 2; ++d) {
         opsf[d] = tail_schedule(m->lt[d], L, true);
         opsv[d] = tail_schedule(m->lt[d], L, false);
         m->nops_f[d] = (int)opsf[d].size();
         m->nops_v[d] = (int)opsv[d].size();
-        if ((e = cudaMalloc(&m->ops_f[d], sizeof(int) * opsf[d].size())) != cudaSuccess) return fail(e);
-        if ((e = cudaMalloc(&m->ops_v[d], sizeof(int) * opsv[d].size())) != cudaSuccess) return fail(e);
     }
-    DevMem phys, msq;
-    if ((e = cudaMalloc(&phys.p, sizeof(double) * np * nmodels)) != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc(&msq.p, sizeof(double))) != cudaSuccess) return fail(e);
+    // every array of the model in one allocation: sized first, then handed out
+    cudaError_t e = cudaSuccess;
+    for (int pass = 0; pass < 2; ++pass) {
+        char* base = static_cast<char*>(m->slab);
+        size_t off = 0;
+        auto take = [&](auto*& q, size_t count) {
+            using E = std::remove_reference_t<decltype(*q)>;
+            if (pass) q = reinterpret_cast<E*>(base + off);
+            off = (off + sizeof(E) * count + 255) & ~size_t(255);
+        };
+        take(m->m_pad, m->n() * nmodels);
+        take(m->lv[0].m2f, m->n() * nmodels);
+        take(m->lv[0].m2d, m->n() * nmodels);
+        if (m->vd) {
+            Level& L0 = m->lv[0];
+            take(L0.rhof, 3 * L0.n());
+            take(L0.rhod, 3 * L0.n());
+            take(L0.gkf, kGalerkinCoefs * L0.n());
+            take(L0.gkd, kGalerkinCoefs * L0.n());
+        }
+        for (int l = 1; l <= L; ++l) {
+            take(m->lv[l].gkf, kGalerkinCoefs * m->lv[l].n() * nmodels);
+            take(m->lv[l].gkd, kGalerkinCoefs * m->lv[l].n() * nmodels);
+        }
+        for (int d = 0; d < 2; ++d) {
+            take(m->ops_f[d], opsf[d].size());
+            take(m->ops_v[d], opsv[d].size());
+        }
+        if (!pass && (e = pool_alloc(ctx, &m->slab, off, s)) != cudaSuccess) return fail(e);
+    }
+    DBuf phys, msq;
+    if ((e = phys.alloc(ctx, sizeof(double) * np * nmodels, s)) != cudaSuccess) return fail(e);
+    if ((e = msq.alloc(ctx, sizeof(double), s)) != cudaSuccess) return fail(e);
     if ((e = cudaMemcpyAsync(phys.p, slowness, sizeof(double) * np * nmodels, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return fail(e);
     for (int d = 0; d < 2; ++d) {
@@ -167,9 +175,9 @@ int create_model(helm_ctx* ctx, cudaStream_t s, int Px, int Pz, double h, const 
             return fail(e);
     }
     launch_pad_model(static_cast<double*>(phys.p), Px, Pz, npml, nmodels, m->m_pad, m->lv[0].m2f, m->lv[0].m2d, s);
-    DevMem rho_phys;
+    DBuf rho_phys;
     if (m->vd) {
-        if ((e = cudaMalloc(&rho_phys.p, sizeof(double) * np)) != cudaSuccess) return fail(e);
+        if ((e = rho_phys.alloc(ctx, sizeof(double) * np, s)) != cudaSuccess) return fail(e);
         if ((e = cudaMemcpyAsync(rho_phys.p, density, sizeof(double) * np, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return fail(e);
         Level& L0 = m->lv[0];
@@ -242,6 +250,7 @@ int helm_ctx_create(int device, void* cuda_stream, helm_ctx** out) {
         c->own_stream = true;
     }
     cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
+    pool_create(c);
     *out = c;
     return HELM_OK;
 }
@@ -252,6 +261,7 @@ void helm_ctx_destroy(helm_ctx* ctx) {
     if (!ctx) return;
     helm_serve_shutdown(ctx);
     DeviceGuard g(ctx->device);
+    pool_destroy(ctx);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -271,19 +281,7 @@ int helm_create_model_rho(helm_ctx* ctx, int Px, int Pz, double h, const double*
 void helm_destroy_model(helm_model* m) {
     if (!m) return;
     DeviceGuard g(m->ctx->device);
-    if (m->m_pad) cudaFree(m->m_pad);
-    for (int d = 0; d < 2; ++d) {
-        if (m->ops_f[d]) cudaFree(m->ops_f[d]);
-        if (m->ops_v[d]) cudaFree(m->ops_v[d]);
-    }
-    for (auto& L : m->lv) {
-        if (L.m2f) cudaFree(L.m2f);
-        if (L.m2d) cudaFree(L.m2d);
-        if (L.gkf) cudaFree(L.gkf);
-        if (L.gkd) cudaFree(L.gkd);
-        if (L.rhof) cudaFree(L.rhof);
-        if (L.rhod) cudaFree(L.rhod);
-    }
+    if (m->slab) cudaFree(m->slab);   // waits for the work that uses it; the memory returns to the context's pool
     delete m;
 }
 
@@ -319,24 +317,24 @@ int helm_solve(helm_model* m, int nrhs, const double* omega, const int* src_ix, 
     cudaStream_t s = m->ctx->stream;
     const size_t n = m->n();
     const size_t fbytes = sizeof(double) * 2 * n * nrhs;
-    DevMem f64, u64, dsrc, fin;
-    if (cudaMalloc(&f64.p, fbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+    DBuf f64, u64, dsrc, fin;
+    if (f64.alloc(m->ctx, fbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
     double* u_dev = nullptr;
     if (o.device_ptrs) {
         u_dev = static_cast<double*>(u_out);
     } else {
-        if (cudaMalloc(&u64.p, fbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+        if (u64.alloc(m->ctx, fbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
         u_dev = static_cast<double*>(u64.p);
     }
     if (!f) {
-        if (cudaMalloc(&dsrc.p, sizeof(int) * nrhs) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+        if (dsrc.alloc(m->ctx, sizeof(int) * nrhs, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
         HELM_CUDA_TRY(cudaMemcpyAsync(dsrc.p, src_flat.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, s));
         launch_point_rhs(static_cast<double*>(f64.p), static_cast<int*>(dsrc.p), nrhs, n, s);
         count_launches(1);
     } else {
         const double* fsrc = static_cast<const double*>(f);
         if (!o.device_ptrs) {
-            if (cudaMalloc(&fin.p, fbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+            if (fin.alloc(m->ctx, fbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
             HELM_CUDA_TRY(cudaMemcpyAsync(fin.p, f, fbytes, cudaMemcpyHostToDevice, s));
             fsrc = static_cast<const double*>(fin.p);
         }
@@ -365,15 +363,15 @@ int helm_apply(helm_model* m, int nrhs, const double* omega, int precision, cons
     cudaStream_t s = m->ctx->stream;
     const bool dbl = precision == HELM_PREC_FP64;
     const size_t bytes = (dbl ? 16 : 8) * m->n() * nrhs;
-    DevMem dw2, du, dy;
+    DBuf dw2, du, dy;
     std::vector<float> w2f(w2.begin(), w2.end());
-    if (cudaMalloc(&dw2.p, sizeof(double) * nrhs) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+    if (dw2.alloc(m->ctx, sizeof(double) * nrhs, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
     if (dbl) HELM_CUDA_TRY(cudaMemcpyAsync(dw2.p, w2.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, s));
     else HELM_CUDA_TRY(cudaMemcpyAsync(dw2.p, w2f.data(), sizeof(float) * nrhs, cudaMemcpyHostToDevice, s));
     const void* up = u;
     void* yp = y;
     if (!device_ptrs) {
-        if (cudaMalloc(&du.p, bytes) != cudaSuccess || cudaMalloc(&dy.p, bytes) != cudaSuccess) {
+        if (du.alloc(m->ctx, bytes, s) != cudaSuccess || dy.alloc(m->ctx, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             return HELM_E_NOMEM;
         }
@@ -436,11 +434,11 @@ int vcycle_call(helm_model* m, int nrhs, const double* omega, double beta1, doub
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
     const size_t bytes = 8 * m->n() * nrhs;
-    DevMem dr, dz;
+    DBuf dr, dz;
     const void* rp = r;
     void* zp = z;
     if (!device_ptrs) {
-        if (cudaMalloc(&dr.p, bytes) != cudaSuccess || cudaMalloc(&dz.p, bytes) != cudaSuccess) {
+        if (dr.alloc(m->ctx, bytes, s) != cudaSuccess || dz.alloc(m->ctx, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             return HELM_E_NOMEM;
         }
@@ -498,15 +496,15 @@ int helm_fwi_forward(helm_model* m, int nfreq, const double* omega, int nshot, c
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
     const size_t dbytes = sizeof(double) * 2 * (size_t)nfreq * nshot * nrec;
-    DevMem dobs, dcal;
+    DBuf dobs, dcal;
     const double* dobs_p = static_cast<const double*>(d_obs);
     double* dcal_p = static_cast<double*>(d_cal_out);
     if (!o.device_ptrs) {
-        if (cudaMalloc(&dobs.p, dbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+        if (dobs.alloc(m->ctx, dbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
         HELM_CUDA_TRY(cudaMemcpyAsync(dobs.p, d_obs, dbytes, cudaMemcpyHostToDevice, s));
         dobs_p = static_cast<const double*>(dobs.p);
         if (d_cal_out) {
-            if (cudaMalloc(&dcal.p, dbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+            if (dcal.alloc(m->ctx, dbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
             dcal_p = static_cast<double*>(dcal.p);
         }
     }
@@ -521,6 +519,7 @@ int helm_fwi_forward(helm_model* m, int nfreq, const double* omega, int nshot, c
     }
     helm_fwi_state* out = new helm_fwi_state();
     out->m = m;
+    out->device = m->ctx->device;
     out->st = st;
     *state = out;
     return rc;
@@ -535,10 +534,10 @@ int helm_fwi_backward(helm_fwi_state* state, double* grad_out, const helm_solve_
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
     const size_t gbytes = sizeof(double) * (size_t)m->Px * m->Pz;
-    DevMem dgrad;
+    DBuf dgrad;
     double* grad_p = grad_out;
     if (!o.device_ptrs) {
-        if (cudaMalloc(&dgrad.p, gbytes) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
+        if (dgrad.alloc(m->ctx, gbytes, s) != cudaSuccess) { cudaGetLastError(); return HELM_E_NOMEM; }
         grad_p = static_cast<double*>(dgrad.p);
     }
     int rc = fwi_backward(state->st, s, grad_p, o, stats);
@@ -560,11 +559,11 @@ int helm_gn_hvp(helm_fwi_state* state, const double* dm, double* hdm_out, const 
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
     const size_t bytes = sizeof(double) * (size_t)m->Px * m->Pz;
-    DevMem ddm, dh;
+    DBuf ddm, dh;
     const double* dm_p = dm;
     double* h_p = hdm_out;
     if (!o.device_ptrs) {
-        if (cudaMalloc(&ddm.p, bytes) != cudaSuccess || cudaMalloc(&dh.p, bytes) != cudaSuccess) {
+        if (ddm.alloc(m->ctx, bytes, s) != cudaSuccess || dh.alloc(m->ctx, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             return HELM_E_NOMEM;
         }
@@ -595,11 +594,11 @@ int helm_gn_step(helm_fwi_state* state, const double* grad, int cg_iters, double
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
     const size_t bytes = sizeof(double) * (size_t)m->Px * m->Pz;
-    DevMem dgrad, ddm;
+    DBuf dgrad, ddm;
     const double* g_p = grad;
     double* dm_p = dm_out;
     if (!o.device_ptrs) {
-        if (cudaMalloc(&dgrad.p, bytes) != cudaSuccess || cudaMalloc(&ddm.p, bytes) != cudaSuccess) {
+        if (dgrad.alloc(m->ctx, bytes, s) != cudaSuccess || ddm.alloc(m->ctx, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             return HELM_E_NOMEM;
         }
@@ -620,7 +619,7 @@ int helm_gn_step(helm_fwi_state* state, const double* grad, int cg_iters, double
 
 void helm_fwi_state_destroy(helm_fwi_state* state) {
     if (!state) return;
-    DeviceGuard g(state->m->ctx->device);
+    DeviceGuard g(state->device);
     fwi_free(state->st);
     delete state;
 }

@@ -85,6 +85,7 @@ struct helm_ctx {
     int num_sms = 0;
     helm::Serve* serve = nullptr;
     std::mutex serve_mu;
+    cudaMemPool_t pool = nullptr;   // workspaces and models (helm_mem.cu)
 };
 
 struct helm_model {
@@ -109,6 +110,7 @@ struct helm_model {
     int tile_restrict[helm::kMaxLevels];
     int tile_prolong[helm::kMaxLevels];
     int tail_level(bool dbl) const { return lt[dbl ? 1 : 0]; }
+    void* slab = nullptr;                 // one device allocation holding every array of the model
     double* m_pad = nullptr;              // device [nmodels][nz][nx] slowness (float64)
     double msq_sum = 0;                   // sum of m^2 over the physical cells
     std::vector<helm::Level> lv;          // lv[0] is the padded fine grid
@@ -116,6 +118,30 @@ struct helm_model {
 };
 
 namespace helm {
+
+// Device memory of a context (helm_mem.cu): a stream-ordered pool of its own, so that the
+// workspace of one call is there for the next one. It keeps at most 1/32 of the device's memory
+// unused between calls and gives all of it back when the context is destroyed, or when any
+// context's allocation on the device does not fit otherwise. Safe with several threads and streams.
+void pool_create(helm_ctx* ctx);
+void pool_destroy(helm_ctx* ctx);
+cudaError_t pool_alloc(helm_ctx* ctx, void** p, size_t bytes, cudaStream_t s);
+size_t pool_unused(helm_ctx* ctx);   // bytes the pool holds that nothing uses
+
+// Stream-ordered device allocation freed on scope exit.
+struct DBuf {
+    void* p = nullptr;
+    cudaStream_t s = nullptr;
+    DBuf() = default;
+    DBuf(const DBuf&) = delete;
+    DBuf& operator=(const DBuf&) = delete;
+    ~DBuf() { if (p) cudaFreeAsync(p, s); }
+    cudaError_t alloc(helm_ctx* ctx, size_t bytes, cudaStream_t st) {
+        s = st;
+        return pool_alloc(ctx, &p, bytes ? bytes : 16, st);
+    }
+    template <typename T> T* as() const { return static_cast<T*>(p); }
+};
 
 // Launch with programmatic stream serialization (the kernel must call pdl_wait
 // before reading anything an earlier kernel of the stream writes).

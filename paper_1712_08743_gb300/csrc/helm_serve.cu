@@ -115,15 +115,16 @@ static int run_batch(helm_ctx* ctx, cudaStream_t s, std::vector<std::shared_ptr<
     int rc = create_model(ctx, s, r0.Px, r0.Pz, r0.h, slow.data(), nb, r0.npml, r0.alpha_max, &m);
     if (rc != HELM_OK) return rc;
     const size_t n = m->n();
-    double *f64 = nullptr, *u64 = nullptr;
-    int* dsrc = nullptr;
+    DBuf f64b, u64b, dsrcb;
     rc = HELM_OK;
-    if (cudaMallocAsync(&f64, sizeof(double) * 2 * n * nb, s) != cudaSuccess ||
-        cudaMallocAsync(&u64, sizeof(double) * 2 * n * nb, s) != cudaSuccess ||
-        cudaMallocAsync(&dsrc, sizeof(int) * nb, s) != cudaSuccess) {
+    if (f64b.alloc(ctx, sizeof(double) * 2 * n * nb, s) != cudaSuccess ||
+        u64b.alloc(ctx, sizeof(double) * 2 * n * nb, s) != cudaSuccess ||
+        dsrcb.alloc(ctx, sizeof(int) * nb, s) != cudaSuccess) {
         cudaGetLastError();
         rc = HELM_E_NOMEM;
     }
+    double *f64 = f64b.as<double>(), *u64 = u64b.as<double>();
+    int* dsrc = dsrcb.as<int>();
     if (rc == HELM_OK && cudaMemcpyAsync(dsrc, src.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, s) != cudaSuccess)
         rc = HELM_E_CUDA;
     if (rc == HELM_OK) {
@@ -137,9 +138,6 @@ static int run_batch(helm_ctx* ctx, cudaStream_t s, std::vector<std::shared_ptr<
                 rc = HELM_E_CUDA;
         }
     }
-    if (f64) cudaFreeAsync(f64, s);
-    if (u64) cudaFreeAsync(u64, s);
-    if (dsrc) cudaFreeAsync(dsrc, s);
     cudaStreamSynchronize(s);
     helm_destroy_model(m);
     return rc;
@@ -165,7 +163,8 @@ static void worker(Serve* sv) {
             cudaMemGetInfo(&fr, &tot);
             const uint64_t cap = sv->budget ? sv->budget : (uint64_t)tot;
             const uint64_t left = cap > sv->in_use ? cap - sv->in_use : 0;
-            avail = sv->budget ? left : std::min<uint64_t>(left, fr);
+            // what the context's pool holds unused is free to this batch as well
+            avail = sv->budget ? left : std::min<uint64_t>(left, fr + pool_unused(sv->ctx));
             avail = avail > sv->reserve ? avail - sv->reserve : 0;
         }
         while (!batch.empty() && batch_bytes(batch[0]->r, (int)batch.size()) > avail) batch.pop_back();

@@ -28,30 +28,44 @@ const char* last_error() { return g_last_error.c_str(); }
 
 namespace {
 
-// Stream-ordered device allocation freed on scope exit.
-struct DBuf {
-    void* p = nullptr;
-    cudaStream_t s = nullptr;
-    DBuf() = default;
-    DBuf(const DBuf&) = delete;
-    DBuf& operator=(const DBuf&) = delete;
-    ~DBuf() { if (p) cudaFreeAsync(p, s); }
-    cudaError_t alloc(size_t bytes, cudaStream_t st) {
-        s = st;
-        return cudaMallocAsync(&p, bytes ? bytes : 16, st);
-    }
-    template <typename T> T* as() const { return static_cast<T*>(p); }
-};
-
+// allocates from the pool of the context of model m (a name in scope where it is used)
+#define TRY_SEND(up, st)                                                                  \
+    do {                                                                                 \
+        cudaError_t e_ = (up).send(m->ctx, (st));                                        \
+        if (e_ != cudaSuccess) {                                                         \
+            cudaGetLastError();                                                          \
+            set_last_error(std::string("upload failed: ") + cudaGetErrorString(e_));     \
+            return e_ == cudaErrorMemoryAllocation ? HELM_E_NOMEM : HELM_E_CUDA;         \
+        }                                                                                \
+    } while (0)
 #define TRY_ALLOC(buf, bytes, st)                                                        \
     do {                                                                                 \
-        cudaError_t e_ = (buf).alloc((bytes), (st));                                     \
+        cudaError_t e_ = (buf).alloc(m->ctx, (bytes), (st));                                   \
         if (e_ != cudaSuccess) {                                                         \
             cudaGetLastError();                                                          \
             set_last_error(std::string("device allocation failed: ") + cudaGetErrorString(e_)); \
             return HELM_E_NOMEM;                                                         \
         }                                                                                \
     } while (0)
+
+// Small host arrays gathered into one host-to-device copy. The host side lives in the object: keep it
+// until the stream has been synchronised.
+struct Upload {
+    std::vector<char> host;
+    DBuf dev;
+    size_t add(const void* src, size_t bytes) {
+        const size_t at = (host.size() + 15) & ~size_t(15);
+        host.resize(at + bytes);
+        std::memcpy(host.data() + at, src, bytes);
+        return at;
+    }
+    template <typename T> size_t add(const std::vector<T>& v) { return add(v.data(), sizeof(T) * v.size()); }
+    cudaError_t send(helm_ctx* ctx, cudaStream_t s) {
+        const cudaError_t e = dev.alloc(ctx, host.size(), s);
+        return e != cudaSuccess ? e : cudaMemcpyAsync(dev.p, host.data(), host.size(), cudaMemcpyHostToDevice, s);
+    }
+    template <typename T> T* at(size_t off) const { return reinterpret_cast<T*>(static_cast<char*>(dev.p) + off); }
+};
 
 int max_blocks_per_rhs(const helm_model* m) {
     const Level& L0 = m->lv[0];
@@ -388,6 +402,7 @@ static void vcycle(const SolveCtx& c, Inner<T>& w, const T* in, T* out, int mode
 // fills fa, its barrier counter and error flag, and points c at it.
 template <typename T>
 static int setup_fcycle(SolveCtx& c, Inner<T>& w, int coarse, DBuf& bar, DBuf& err, FcArgs* fa) {
+    const helm_model* m = c.m;
     c.fca = nullptr;
     if constexpr (sizeof(T) == 4) {
         if (coarse != HELM_COARSE_FUSED || c.ld <= 0) return HELM_OK;
@@ -450,6 +465,7 @@ static int alloc_levels(const helm_model* m, cudaStream_t s, int nrhs, Inner<T>&
 
 template <typename T>
 static int alloc_inner(const SolveCtx& c, Inner<T>& w) {
+    const helm_model* m = c.m;
     const size_t n = c.m->n(), vb = sizeof(T) * 2 * n * c.nrhs;
     TRY_ALLOC(w.x, vb, c.s);
     if (c.o.krylov == HELM_KRYLOV_BICGSTAB) {      // FGMRES keeps its vectors in FgBufs
@@ -509,10 +525,16 @@ static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, cudaGraphEx
                             c.nrhs, c.s);
     NvtxRange nv("bicgstab inner solve");
     const int chunk = std::max(1, c.o.check_every);
+    // The graph holds the largest part of a chunk up to five iterations and is launched until the
+    // chunk is done: a node costs about 3.7 us to instantiate (ten iterations of 21 kernels: 0.8 ms of
+    // a 6 ms solve), a launch about 19 us of idle GPU; for the 40 to 60 iterations of a small
+    // solve the sum is least between three and five iterations.
+    int per_graph = std::min(chunk, 5);
+    while (chunk % per_graph) --per_graph;
     if (c.o.use_graphs && *graph == nullptr) {
         cudaGraph_t g;
         HELM_CUDA_TRY(cudaStreamBeginCapture(c.s, cudaStreamCaptureModeThreadLocal));
-        for (int k = 0; k < chunk; ++k) bicg_iteration<T>(c, w);
+        for (int k = 0; k < per_graph; ++k) bicg_iteration<T>(c, w);
         cudaError_t e = cudaStreamEndCapture(c.s, &g);
         if (e != cudaSuccess) { set_last_error(cudaGetErrorString(e)); return HELM_E_CUDA; }
         e = cudaGraphInstantiate(graph, g, 0);
@@ -532,7 +554,7 @@ static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, cudaGraphEx
     if (guard_iters > 0) hs.resize(c.nrhs);
     while (done < limit) {
         if (c.o.use_graphs) {
-            HELM_CUDA_TRY(cudaGraphLaunch(*graph, c.s));
+            for (int k = 0; k < chunk; k += per_graph) HELM_CUDA_TRY(cudaGraphLaunch(*graph, c.s));
         } else {
             for (int k = 0; k < chunk; ++k) bicg_iteration<T>(c, w);
         }
@@ -569,20 +591,21 @@ struct FgBufs {
 
 template <typename T>
 static int alloc_fg(const SolveCtx& c, FgBufs<T>& f) {
-    const int m = c.o.restart, nrhs = c.nrhs;
+    const helm_model* m = c.m;
+    const int mr = c.o.restart, nrhs = c.nrhs;
     const size_t vb = sizeof(T) * 2 * c.m->n() * nrhs;
-    TRY_ALLOC(f.V, vb * (m + 1), c.s);
-    TRY_ALLOC(f.Z, vb * m, c.s);
-    TRY_ALLOC(f.H, sizeof(double2) * (size_t)nrhs * (m + 1) * m, c.s);
-    TRY_ALLOC(f.g, sizeof(double2) * (size_t)nrhs * (m + 1), c.s);
-    TRY_ALLOC(f.cs, sizeof(double) * (size_t)nrhs * m, c.s);
-    TRY_ALLOC(f.sn, sizeof(double2) * (size_t)nrhs * m, c.s);
-    TRY_ALLOC(f.y, sizeof(double2) * (size_t)nrhs * m, c.s);
-    TRY_ALLOC(f.tmp, sizeof(double2) * (size_t)nrhs * (m + 1), c.s);
-    TRY_ALLOC(f.sc, sizeof(double) * (size_t)nrhs * (m + 1), c.s);
+    TRY_ALLOC(f.V, vb * (mr + 1), c.s);
+    TRY_ALLOC(f.Z, vb * mr, c.s);
+    TRY_ALLOC(f.H, sizeof(double2) * (size_t)nrhs * (mr + 1) * mr, c.s);
+    TRY_ALLOC(f.g, sizeof(double2) * (size_t)nrhs * (mr + 1), c.s);
+    TRY_ALLOC(f.cs, sizeof(double) * (size_t)nrhs * mr, c.s);
+    TRY_ALLOC(f.sn, sizeof(double2) * (size_t)nrhs * mr, c.s);
+    TRY_ALLOC(f.y, sizeof(double2) * (size_t)nrhs * mr, c.s);
+    TRY_ALLOC(f.tmp, sizeof(double2) * (size_t)nrhs * (mr + 1), c.s);
+    TRY_ALLOC(f.sc, sizeof(double) * (size_t)nrhs * (mr + 1), c.s);
     TRY_ALLOC(f.wn2, sizeof(double) * (size_t)nrhs, c.s);
-    HELM_CUDA_TRY(cudaMemsetAsync(f.H.p, 0, sizeof(double2) * (size_t)nrhs * (m + 1) * m, c.s));
-    f.dev.m = m;
+    HELM_CUDA_TRY(cudaMemsetAsync(f.H.p, 0, sizeof(double2) * (size_t)nrhs * (mr + 1) * mr, c.s));
+    f.dev.m = mr;
     f.dev.H = f.H.template as<double2>();
     f.dev.g = f.g.template as<double2>();
     f.dev.cs = f.cs.template as<double>();
@@ -680,8 +703,11 @@ static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* r
 // inverse of the coarsest level that the shared-memory tail uses (FP32 and FP64
 // copies). One inverse per distinct (model, frequency) pair: slot[b].
 struct CoarseSet {
-    DBuf work, mf, md, slot, w2s, mods;
-    DBuf grp, err;                     // dense path
+    DBuf work, mf, md;
+    DBuf err;                          // dense path: set by the inversion (coarse_failed)
+    Upload up;                         // slot, w2s, mods and (dense path) grp
+    const int* slot = nullptr;
+    const int* grp = nullptr;
     int n = 0, nslots = 0;
     int ld = 0;                        // > 0: the dense path, level ld
     int ngroups = 0, maxg = 0;
@@ -710,13 +736,6 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
         slot[b] = it->second;
     }
     cs.nslots = (int)w2s.size();
-    TRY_ALLOC(cs.slot, sizeof(int) * nrhs, s);
-    TRY_ALLOC(cs.w2s, sizeof(double) * cs.nslots, s);
-    TRY_ALLOC(cs.mods, sizeof(int) * cs.nslots, s);
-    HELM_CUDA_TRY(cudaMemcpyAsync(cs.slot.p, slot.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpyAsync(cs.w2s.p, w2s.data(), sizeof(double) * cs.nslots, cudaMemcpyHostToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpyAsync(cs.mods.p, mods.data(), sizeof(int) * cs.nslots, cudaMemcpyHostToDevice, s));
-
     const bool want_dense = coarse == HELM_COARSE_DENSE || coarse == HELM_COARSE_FUSED ||
                             (coarse == HELM_COARSE_AUTO && nrhs <= kDenseAutoMaxRhs);
     if (want_dense && b2 != 0.0 && m->ld > 0 && dense_invert_fits(m->lv[m->ld].nx, m->lv[m->ld].nz)) {
@@ -733,26 +752,24 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
         DBuf& mi = dbl ? cs.md : cs.mf;
         TRY_ALLOC(mi, es * (size_t)n * n * cs.nslots, s);
         TRY_ALLOC(cs.err, sizeof(int), s);
-        TRY_ALLOC(cs.grp, sizeof(int) * grp.size(), s);
-        HELM_CUDA_TRY(cudaMemcpyAsync(cs.grp.p, grp.data(), sizeof(int) * grp.size(), cudaMemcpyHostToDevice, s));
+        const size_t o_slot = cs.up.add(slot), o_w2s = cs.up.add(w2s), o_mods = cs.up.add(mods), o_grp = cs.up.add(grp);
+        TRY_SEND(cs.up, s);
+        const double* w2s_d = cs.up.at<double>(o_w2s);
+        const int* mods_d = cs.up.at<int>(o_mods);
         const LevelDev Ld = level_dev(m, ld, true);
-        cudaError_t e = dbl ? launch_dense_invert<double>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1,
-                                                          b2, cs.md.as<double>(), cs.err.as<int>(), s)
-                            : launch_dense_invert<float>(Ld, cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots, b1,
-                                                         b2, cs.mf.as<float>(), cs.err.as<int>(), s);
-        int herr = -1;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, cs.err.p, sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && herr == 0) {
-            cs.ld = ld;
-            cs.n = n;
-            cs.ngroups = (int)grp.size() - 1;
-            cs.maxg = maxg;
-            return HELM_OK;
-        }
-        // the dense inverse could not be formed (a failed launch, or a
-        // vanishing pivot): fall back to the multigrid tail below
-        cudaGetLastError();
+        const cudaError_t e =
+            dbl ? launch_dense_invert<double>(Ld, w2s_d, mods_d, cs.nslots, b1, b2, cs.md.as<double>(),
+                                              cs.err.as<int>(), s)
+                : launch_dense_invert<float>(Ld, w2s_d, mods_d, cs.nslots, b1, b2, cs.mf.as<float>(),
+                                             cs.err.as<int>(), s);
+        HELM_CUDA_TRY(e);
+        cs.slot = cs.up.at<int>(o_slot);
+        cs.grp = cs.up.at<int>(o_grp);
+        cs.ld = ld;
+        cs.n = n;
+        cs.ngroups = (int)grp.size() - 1;
+        cs.maxg = maxg;
+        return HELM_OK;
     }
 
     const Level& Lc = m->lv.back();
@@ -762,12 +779,26 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
     TRY_ALLOC(cs.work, sizeof(double2) * nn * 2 * cs.nslots, s);
     TRY_ALLOC(cs.mf, sizeof(float2) * nn * cs.nslots, s);
     TRY_ALLOC(cs.md, sizeof(double2) * nn * cs.nslots, s);
+    const size_t o_slot = cs.up.add(slot), o_w2s = cs.up.add(w2s), o_mods = cs.up.add(mods);
+    TRY_SEND(cs.up, s);
+    cs.slot = cs.up.at<int>(o_slot);
     count_launches(1);
-    launch_coarse_invert(level_dev(m, (int)m->lv.size() - 1, true), cs.w2s.as<double>(), cs.mods.as<int>(), cs.nslots,
-                         b1, b2, cs.work.as<double2>(), cs.mf.as<float2>(), cs.md.as<double2>(), s);
+    launch_coarse_invert(level_dev(m, (int)m->lv.size() - 1, true), cs.up.at<double>(o_w2s), cs.up.at<int>(o_mods),
+                         cs.nslots, b1, b2, cs.work.as<double2>(), cs.mf.as<float2>(), cs.md.as<double2>(), s);
     HELM_CUDA_TRY(cudaGetLastError());
-    // the host vectors above must outlive the copies
+    return HELM_OK;
+}
+
+// Whether the dense inverse could not be formed (a vanishing pivot): the caller then builds the
+// multigrid tail's inverse in its place. Waits for the stream, so it is asked where the caller
+// waits anyway: the work that uses the inverse is already in the stream behind it.
+static int coarse_failed(const CoarseSet& cs, cudaStream_t s, bool* failed) {
+    *failed = false;
+    if (cs.ld <= 0) return HELM_OK;
+    int h = 0;
+    HELM_CUDA_TRY(cudaMemcpyAsync(&h, cs.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     HELM_CUDA_TRY(cudaStreamSynchronize(s));
+    *failed = h != 0;
     return HELM_OK;
 }
 
@@ -785,10 +816,14 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
     c.pstride = 3 * max_blocks_per_rhs(m);
     if (o.krylov == HELM_KRYLOV_FGMRES) c.pstride = std::max(c.pstride, fg_partials(m->n()));
     c.lf = fcycle_level(m, h_w2, nrhs);
-    DBuf w2, w2f, st, part, nact, rin;
-    TRY_ALLOC(w2, sizeof(double) * nrhs, s);
-    TRY_ALLOC(w2f, sizeof(float) * nrhs, s);
-    TRY_ALLOC(st, sizeof(RhsState) * nrhs, s);
+    std::vector<RhsState> hs(nrhs);
+    std::memset(hs.data(), 0, sizeof(RhsState) * nrhs);
+    for (auto& S : hs) { S.outer_active = 1; S.active = 1; S.max_it = o.max_it; }
+    Upload up;
+    const size_t o_st = up.add(hs), o_w2 = up.add(h_w2, sizeof(double) * nrhs);
+    const size_t o_w2f = up.add(std::vector<float>(h_w2, h_w2 + nrhs));
+    TRY_SEND(up, s);
+    DBuf part, nact, rin;
     TRY_ALLOC(part, sizeof(double) * (size_t)c.pstride * nrhs, s);
     TRY_ALLOC(nact, sizeof(int), s);
     TRY_ALLOC(rin, sizeof(T) * 2 * n * nrhs, s);
@@ -796,17 +831,17 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
     std::unique_ptr<CoarseSet> cs(new CoarseSet());
     int rc = build_coarse(m, s, nrhs, h_w2, o.beta1, o.beta2, sizeof(T) == 8, coarse, *cs);
     if (rc != HELM_OK) return rc;
-    c.w2 = w2.as<double>();
-    c.w2f = w2f.as<float>();
-    c.st = st.as<RhsState>();
+    c.w2 = up.at<double>(o_w2);
+    c.w2f = up.at<float>(o_w2f);
+    c.st = up.at<RhsState>(o_st);
     c.partials = part.as<double>();
     c.nactive = nact.as<int>();
     auto use_coarse = [&](const CoarseSet& q) {
-        c.slot = q.slot.as<int>();
+        c.slot = q.slot;
         c.ncoarse = q.n;
         c.minv = q.minv(sizeof(T) == 8);
         c.ld = q.ld;
-        c.grp = q.grp.as<int>();
+        c.grp = q.grp;
         c.ngroups = q.ngroups;
         c.maxg = q.maxg;
     };
@@ -832,13 +867,6 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         if (rc != HELM_OK) return rc;
     }
 
-    std::vector<RhsState> hs(nrhs);
-    std::memset(hs.data(), 0, sizeof(RhsState) * nrhs);
-    for (auto& S : hs) { S.outer_active = 1; S.active = 1; S.max_it = o.max_it; }
-    HELM_CUDA_TRY(cudaMemcpyAsync(c.st, hs.data(), sizeof(RhsState) * nrhs, cudaMemcpyHostToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpyAsync(w2.p, h_w2, sizeof(double) * nrhs, cudaMemcpyHostToDevice, s));
-    std::vector<float> h_w2f(h_w2, h_w2 + nrhs);
-    HELM_CUDA_TRY(cudaMemcpyAsync(w2f.p, h_w2f.data(), sizeof(float) * nrhs, cudaMemcpyHostToDevice, s));
     HELM_CUDA_TRY(cudaMemsetAsync(part.p, 0, sizeof(double) * (size_t)c.pstride * nrhs, s));
     HELM_CUDA_TRY(cudaMemsetAsync(u64, 0, sizeof(double) * 2 * n * nrhs, s));
 
@@ -878,6 +906,21 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         for (int b = 0; b < nrhs; ++b)
             if (hs[b].outer_active) { any = 1; }
         if (!any || outer >= max_outer) break;
+        if (outer == 0) {
+            // the level vectors go down to the dense level, so to the tail's first level too
+            bool failed = false;
+            rc = coarse_failed(*cs, s, &failed);
+            if (rc == HELM_OK && failed) {
+                std::unique_ptr<CoarseSet> cs2(new CoarseSet());
+                rc = build_coarse(m, s, nrhs, h_w2, o.beta1, o.beta2, sizeof(T) == 8, HELM_COARSE_TAIL, *cs2);
+                if (rc == HELM_OK) {
+                    cs.swap(cs2);
+                    use_coarse(*cs);
+                    rc = setup_fcycle<T>(c, w, coarse, fcbar, fcerr, fca.get());
+                }
+            }
+            if (rc != HELM_OK) break;
+        }
         if (guard && !switched) {
             bool stall = force_switch;
             for (int b = 0; b < nrhs; ++b) {
@@ -894,6 +937,13 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
                 c.o.beta2 = 1.0;
                 std::unique_ptr<CoarseSet> cs2(new CoarseSet());
                 rc = build_coarse(m, s, nrhs, h_w2, 1.0, 1.0, sizeof(T) == 8, coarse, *cs2);
+                if (rc != HELM_OK) break;
+                bool failed = false;
+                rc = coarse_failed(*cs2, s, &failed);
+                if (rc == HELM_OK && failed) {
+                    cs2.reset(new CoarseSet());
+                    rc = build_coarse(m, s, nrhs, h_w2, 1.0, 1.0, sizeof(T) == 8, HELM_COARSE_TAIL, *cs2);
+                }
                 if (rc != HELM_OK) break;
                 cs.swap(cs2);
                 use_coarse(*cs);
@@ -967,25 +1017,23 @@ int vcycle_once(const helm_model* m, cudaStream_t s, int nrhs, const double* h_w
     c.o.omega_jacobi = wj;
     c.pstride = 3 * max_blocks_per_rhs(m);
     c.lf = fcycle_level(m, h_w2, nrhs);
-    DBuf w2, w2f;
-    TRY_ALLOC(w2, sizeof(double) * nrhs, s);
-    TRY_ALLOC(w2f, sizeof(float) * nrhs, s);
-    HELM_CUDA_TRY(cudaMemcpyAsync(w2.p, h_w2, sizeof(double) * nrhs, cudaMemcpyHostToDevice, s));
-    std::vector<float> h_w2f(h_w2, h_w2 + nrhs);
-    HELM_CUDA_TRY(cudaMemcpyAsync(w2f.p, h_w2f.data(), sizeof(float) * nrhs, cudaMemcpyHostToDevice, s));
+    Upload up;
+    const size_t o_w2 = up.add(h_w2, sizeof(double) * nrhs);
+    const size_t o_w2f = up.add(std::vector<float>(h_w2, h_w2 + nrhs));
+    TRY_SEND(up, s);
     CoarseSet cs;
     int rc = build_coarse(m, s, nrhs, h_w2, b1, b2, false, coarse, cs);
     if (rc != HELM_OK) return rc;
-    c.w2 = w2.as<double>();
-    c.w2f = w2f.as<float>();
+    c.w2 = up.at<double>(o_w2);
+    c.w2f = up.at<float>(o_w2f);
     c.st = nullptr;
     c.partials = nullptr;
     c.nactive = nullptr;
-    c.slot = cs.slot.as<int>();
+    c.slot = cs.slot;
     c.ncoarse = cs.n;
     c.minv = cs.mf.p;
     c.ld = cs.ld;
-    c.grp = cs.grp.as<int>();
+    c.grp = cs.grp;
     c.ngroups = cs.ngroups;
     c.maxg = cs.maxg;
     Inner<float> w;
@@ -997,6 +1045,10 @@ int vcycle_once(const helm_model* m, cudaStream_t s, int nrhs, const double* h_w
     if (rc != HELM_OK) return rc;
     vcycle<float>(c, w, r, z, 0, nullptr, nullptr);
     HELM_CUDA_TRY(cudaGetLastError());
+    bool failed = false;
+    rc = coarse_failed(cs, s, &failed);
+    if (rc != HELM_OK) return rc;
+    if (failed) return vcycle_once(m, s, nrhs, h_w2, b1, b2, wj, HELM_COARSE_TAIL, r, z);
     HELM_CUDA_TRY(cudaStreamSynchronize(s));
     return check_fcycle(c, fcerr);
 }
@@ -1268,7 +1320,7 @@ int fwi_forward(const helm_model* m, cudaStream_t s, int nfreq, const double* om
             src[f * nshot + k] = src_flat_h[k];
         }
     auto am = [&](void** p, size_t b) {
-        if (cudaMalloc(p, b ? b : 16) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (pool_alloc(m->ctx, p, b ? b : 16, s) != cudaSuccess) { cudaGetLastError(); return false; }
         return true;
     };
     if (!am((void**)&st->u64, sizeof(double) * 2 * n * nrhs) || !am((void**)&st->resid, sizeof(double) * 2 * (size_t)nrec * nrhs) ||
