@@ -115,10 +115,9 @@ __device__ __forceinline__ cx<T> mop9_staged(const GalTile<T, W, H>& t, int nx, 
     return acc;
 }
 
-// Default tiles of the Galerkin kernels: restriction coarse tile RCX x RCZ,
-// prolongation fine tile PX x PZ; halved in x for complex128 to stay within 48 KB
-// of static shared memory. The complex64 kernels also come in the other shapes of
-// kGalTiles (helm_kernels.cu), among which the autotuner chooses per level.
+// complex128 tiles of the Galerkin kernels (restriction coarse tile RCX x RCZ, prolongation fine tile PX x PZ),
+// within 48 KB of static shared memory. The complex64 kernels come in several shapes
+// (helm_kernels.cu), chosen by the level's size or by the autotuner.
 template <typename T> struct GTile {
     static constexpr int RCX = sizeof(T) == 4 ? 16 : 8, RCZ = 8;
     static constexpr int PX = sizeof(T) == 4 ? 32 : 16, PZ = 8;
@@ -337,30 +336,31 @@ __device__ __forceinline__ void resid_restrict_tile_work(ResidRestrictTile<T, GR
 // Fine tile (x0, z0) of GPX x GPZ nodes, GPX * GPZ threads: u = wj D^-1 f + P e
 // on the tile and its halo, then the post-smoothing sweep u + wj D^-1 (f - M u),
 // written to out (added to it when accumulating).
-template <typename T, int GPX, int GPZ_ = GTile<T>::PZ>
+template <typename T, int GPX, int GPZ_ = GTile<T>::PZ, int NT_ = GPX * GPZ_>
 struct ProlongTile {
     static constexpr int GPZ = GPZ_;
     static constexpr int RW = GPX + 2, RH = GPZ + 2;
     static constexpr int EW = GPX / 2 + 2, EH = GPZ / 2 + 2;
-    static constexpr int NT = GPX * GPZ;
+    static constexpr int NT = NT_;   // threads of the tile (more than its nodes spreads the halo)
+    static_assert(NT >= GPX * GPZ, "one thread per node at least");
     GalTile<T, RW, RH> C;
     cx<T> F[RH][RW];
     cx<T> U2[RH][RW];
     cx<T> E[EH][EW];
 };
 
-template <typename T, int GPX, int GPZ>
-__device__ __forceinline__ void prolong_tile_stage(ProlongTile<T, GPX, GPZ>& sm, const LevelDev& Lf, int bx, int by,
+template <typename T, int GPX, int GPZ, int NT_ = GPX * GPZ>
+__device__ __forceinline__ void prolong_tile_stage(ProlongTile<T, GPX, GPZ, NT_>& sm, const LevelDev& Lf, int bx, int by,
                                                    int b, T hw, T b1, T b2, int tid) {
-    using PT = ProlongTile<T, GPX, GPZ>;
+    using PT = ProlongTile<T, GPX, GPZ, NT_>;
     stage_gal<T, PT::RW, PT::RH, PT::NT>(sm.C, Lf, b, hw * b1, hw * b2, bx * GPX - 1, by * PT::GPZ - 1, tid);
 }
 
-template <typename T, int GPX, int GPZ, bool COH, class Sync>
-__device__ __forceinline__ void prolong_tile_work(ProlongTile<T, GPX, GPZ>& sm, const LevelDev& Lf, const LevelDev& Lc,
+template <typename T, int GPX, int GPZ, bool COH, class Sync, int NT_ = GPX * GPZ>
+__device__ __forceinline__ void prolong_tile_work(ProlongTile<T, GPX, GPZ, NT_>& sm, const LevelDev& Lf, const LevelDev& Lc,
                                                   T wj, const T* f, const T* ec, T* out, int accumulate, int bx,
                                                   int by, int b, int tid, Sync sync) {
-    using PT = ProlongTile<T, GPX, GPZ>;
+    using PT = ProlongTile<T, GPX, GPZ, NT_>;
     constexpr int RW = PT::RW, RH = PT::RH, EW = PT::EW, EH = PT::EH;
     const int x0 = bx * GPX, z0 = by * GPZ;
     const int gx0 = x0 - 1, gz0 = z0 - 1;
@@ -385,7 +385,7 @@ __device__ __forceinline__ void prolong_tile_work(ProlongTile<T, GPX, GPZ>& sm, 
     cx<T> opre(0, 0);
     {
         const int tz = tid / GPX, tx = tid - tz * GPX;
-        if (accumulate && x0 + tx < Lf.nx && z0 + tz < Lf.nz) {
+        if (accumulate && tz < GPZ && x0 + tx < Lf.nx && z0 + tz < Lf.nz) {
             const size_t i = (size_t)(z0 + tz) * Lf.nx + x0 + tx;
             opre = COH ? ldv<true>(ob, i) : ldcc(ob, i);
         }
@@ -422,7 +422,7 @@ __device__ __forceinline__ void prolong_tile_work(ProlongTile<T, GPX, GPZ>& sm, 
     sync();
     const int tz = tid / GPX, tx = tid - tz * GPX;   // one output point per thread
     const int gx = x0 + tx, gz = z0 + tz;
-    if (gx < Lf.nx && gz < Lf.nz) {
+    if (tz < GPZ && gx < Lf.nx && gz < Lf.nz) {
         const int lx = tx + 1, lz = tz + 1;
         const size_t i = (size_t)gz * Lf.nx + gx;
         const cx<T> c = sm.U2[lz][lx];
@@ -441,9 +441,9 @@ __device__ __forceinline__ void prolong_tile_work(ProlongTile<T, GPX, GPZ>& sm, 
 // one, then u2 + wj D^-1 (f - M u2) (added to the level's previous correction when
 // acc_m). Each node's arithmetic is the one-level tile's, so the result is that of
 // the two launches; level l + 1's correction is not written (nothing reads it).
-template <typename T, int GPX, int GPZ>
+template <typename T, int GPX, int GPZ, int NT_ = GPX * GPZ>
 struct Prolong2Tile {
-    using PT = ProlongTile<T, GPX, GPZ>;
+    using PT = ProlongTile<T, GPX, GPZ, NT_>;
     static constexpr int EW = PT::EW, EH = PT::EH;            // level l + 1 nodes the level l tile reads
     static constexpr int MW = EW + 2, MH = EH + 2;            // their u2 region
     static constexpr int CW = EW / 2 + 3, CH = EH / 2 + 3;    // level l + 2 footprint of that region (bound)
@@ -454,25 +454,25 @@ struct Prolong2Tile {
     cx<T> CE[CH][CW];
 };
 
-template <typename T, int GPX, int GPZ>
-__device__ __forceinline__ void prolong2_tile_stage(Prolong2Tile<T, GPX, GPZ>& sm, const LevelDev& Lf,
+template <typename T, int GPX, int GPZ, int NT_ = GPX * GPZ>
+__device__ __forceinline__ void prolong2_tile_stage(Prolong2Tile<T, GPX, GPZ, NT_>& sm, const LevelDev& Lf,
                                                     const LevelDev& Lm, int bx, int by, int b, T hw, T b1, T b2,
                                                     int tid) {
-    using P2 = Prolong2Tile<T, GPX, GPZ>;
-    prolong_tile_stage<T, GPX, GPZ>(sm.fine, Lf, bx, by, b, hw, b1, b2, tid);
+    using P2 = Prolong2Tile<T, GPX, GPZ, NT_>;
+    prolong_tile_stage<T, GPX, GPZ, NT_>(sm.fine, Lf, bx, by, b, hw, b1, b2, tid);
     const int ax0 = bx * GPX / 2 - 1, az0 = by * GPZ / 2 - 1;
-    stage_gal<T, P2::MW, P2::MH, GPX * GPZ>(sm.MC, Lm, b, hw * b1, hw * b2, ax0 - 1, az0 - 1, tid);
+    stage_gal<T, P2::MW, P2::MH, NT_>(sm.MC, Lm, b, hw * b1, hw * b2, ax0 - 1, az0 - 1, tid);
 }
 
 // fl, fm: right-hand sides of levels l and l + 1; ec: correction of level l + 2;
 // out: level l's correction (added to when acc_f); em: level l + 1's previous
 // correction (added when acc_m).
-template <typename T, int GPX, int GPZ, bool COH, class Sync>
-__device__ __forceinline__ void prolong2_tile_work(Prolong2Tile<T, GPX, GPZ>& sm, const LevelDev& Lf,
+template <typename T, int GPX, int GPZ, bool COH, class Sync, int NT_ = GPX * GPZ>
+__device__ __forceinline__ void prolong2_tile_work(Prolong2Tile<T, GPX, GPZ, NT_>& sm, const LevelDev& Lf,
                                                    const LevelDev& Lm, const LevelDev& Lc, T wj, const T* fl,
                                                    const T* fm, const T* ec, const T* em, T* out, int acc_f,
                                                    int acc_m, int bx, int by, int b, int tid, Sync sync) {
-    using P2 = Prolong2Tile<T, GPX, GPZ>;
+    using P2 = Prolong2Tile<T, GPX, GPZ, NT_>;
     using PT = typename P2::PT;
     constexpr int NT = PT::NT, RW = PT::RW, RH = PT::RH, EW = P2::EW, EH = P2::EH;
     constexpr int MW = P2::MW, MH = P2::MH, CW = P2::CW, CH = P2::CH;
@@ -507,7 +507,7 @@ __device__ __forceinline__ void prolong2_tile_work(Prolong2Tile<T, GPX, GPZ>& sm
     cx<T> opre(0, 0);
     {
         const int tz = tid / GPX, tx = tid - tz * GPX;
-        if (acc_f && x0 + tx < Lf.nx && z0 + tz < Lf.nz) {
+        if (acc_f && tz < GPZ && x0 + tx < Lf.nx && z0 + tz < Lf.nz) {
             const size_t i = (size_t)(z0 + tz) * Lf.nx + x0 + tx;
             opre = COH ? ldv<true>(ob, i) : ldcc(ob, i);
         }
@@ -601,7 +601,7 @@ __device__ __forceinline__ void prolong2_tile_work(Prolong2Tile<T, GPX, GPZ>& sm
     sync();
     const int tz = tid / GPX, tx = tid - tz * GPX;
     const int gx = x0 + tx, gz = z0 + tz;
-    if (gx < Lf.nx && gz < Lf.nz) {
+    if (tz < GPZ && gx < Lf.nx && gz < Lf.nz) {
         const int lx = tx + 1, lz = tz + 1;
         const size_t i = (size_t)gz * Lf.nx + gx;
         const cx<T> c = sm.fine.U2[lz][lx];

@@ -903,17 +903,17 @@ __global__ void __launch_bounds__(NT) k_restrict_g(LevelDev Lf, LevelDev Lc, con
                                                           threadIdx.x, BlockSync{});
 }
 
-template <typename T, int GPX, int GPZ>
-__global__ void __launch_bounds__(GPX * GPZ) k_prolong_g(LevelDev Lf, LevelDev Lc, const T* __restrict__ hwv, T b1,
+template <typename T, int GPX, int GPZ, int NT = GPX * GPZ>
+__global__ void __launch_bounds__(NT) k_prolong_g(LevelDev Lf, LevelDev Lc, const T* __restrict__ hwv, T b1,
                                                          T b2, T wj, const T* __restrict__ f, const T* __restrict__ ec,
                                                          T* __restrict__ out, const RhsState* st, int accumulate) {
-    __shared__ ProlongTile<T, GPX, GPZ> sm;
+    __shared__ ProlongTile<T, GPX, GPZ, NT> sm;
     pdl_trigger();
     const int b = blockIdx.z;
-    prolong_tile_stage<T, GPX, GPZ>(sm, Lf, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);   // model data
+    prolong_tile_stage<T, GPX, GPZ, NT>(sm, Lf, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);   // model data
     pdl_wait();
     if (!rhs_active(st, b)) return;
-    prolong_tile_work<T, GPX, GPZ, false>(sm, Lf, Lc, wj, f, ec, out, accumulate, blockIdx.x, blockIdx.y, b,
+    prolong_tile_work<T, GPX, GPZ, false, BlockSync, NT>(sm, Lf, Lc, wj, f, ec, out, accumulate, blockIdx.x, blockIdx.y, b,
                                           threadIdx.x, BlockSync{});
 }
 
@@ -933,6 +933,20 @@ __global__ void __launch_bounds__(NT) k_resid_restrict_g(LevelDev Lf, LevelDev L
     resid_restrict_tile_work<T, GRCX, GRCZ, NT, false>(sm, Lf, Lc, wj, f, e, g, fc, blockIdx.x, blockIdx.y, b,
                                                        threadIdx.x, BlockSync{});
 }
+
+// Whether a Galerkin level is small for the GPU: its restriction's coarse nodes, over the batch
+// (at most kGalMarchMinRhs right-hand sides), fill less than about one wave of tiles. What counts
+// there is the chain of one tile (loads, smoothing, stencil, weights, four barriers), so
+// the tiles are small and every fine node of a tile has a thread of its own; above it the
+// halo's repeated work counts and the tiles are larger. Measured on whole solves (ms, all levels
+// 16 x 8 tiles on 128 threads -> this rule): 1041 x 1041 with one right-hand side 256.5 -> 227 (of
+// its levels, 260 x 260 coarse nodes prefer 8 x 16 tiles by 1.5 %, 130 x 130 and below 8 x 4 by 1 to
+// 2 %), 141 x 141 5.22 -> 4.70, five on 213 x 137 12.5 -> 11.8, four on 341 x 191 15.9 -> 15.3.
+constexpr double kSmallLevelNodes = 32768.0;
+// Prolongation tiles (one thread per node): 16 x 8 below, 32 x 8 above.
+constexpr double kSmallProlongNodes = 1e6;
+inline bool small_prolong(const LevelDev& Lf, int nrhs) { return (double)Lf.nx * Lf.nz * nrhs <= kSmallProlongNodes; }
+inline bool small_level(const LevelDev& Lc, int nrhs) { return (double)Lc.nx * Lc.nz * nrhs <= kSmallLevelNodes; }
 
 template <typename T, int GRCX, int GRCZ, int NT>
 static void launch_resid_restrict_shape(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double b1, double b2,
@@ -954,10 +968,12 @@ void launch_resid_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, 
     if constexpr (sizeof(T) == 4) {
         if (tile == 0)
             launch_resid_restrict_shape<T, 8, 8, 64>(Lf, Lc, w2, b1, b2, wj, f, e, g, fc, st, nrhs, s);
+        else if (tile == 1 && small_level(Lc, nrhs))
+            launch_resid_restrict_shape<T, 8, 4, 288>(Lf, Lc, w2, b1, b2, wj, f, e, g, fc, st, nrhs, s);
         else
             launch_resid_restrict_shape<T, 8, 8, 128>(Lf, Lc, w2, b1, b2, wj, f, e, g, fc, st, nrhs, s);
     } else {
-        launch_resid_restrict_shape<T, 8, 4, 64>(Lf, Lc, w2, b1, b2, wj, f, e, g, fc, st, nrhs, s);
+        launch_resid_restrict_shape<T, 8, 4, 288>(Lf, Lc, w2, b1, b2, wj, f, e, g, fc, st, nrhs, s);
     }
 }
 template void launch_resid_restrict<float>(const LevelDev&, const LevelDev&, const float*, double, double, double,
@@ -969,28 +985,28 @@ template void launch_resid_restrict<double>(const LevelDev&, const LevelDev&, co
 
 // two prolongations in one launch (tile body prolong2_tile_work): level l + 1's
 // from e of level l + 2, then level l's
-template <typename T, int GPX, int GPZ>
-__global__ void __launch_bounds__(GPX * GPZ) k_prolong2_g(LevelDev Lf, LevelDev Lm, LevelDev Lc,
+template <typename T, int GPX, int GPZ, int NT = GPX * GPZ>
+__global__ void __launch_bounds__(NT) k_prolong2_g(LevelDev Lf, LevelDev Lm, LevelDev Lc,
                                                           const T* __restrict__ hwv, T b1, T b2, T wj,
                                                           const T* __restrict__ fl, const T* __restrict__ fm,
                                                           const T* __restrict__ ec, const T* em, T* out,
                                                           const RhsState* st, int acc_f, int acc_m) {
-    __shared__ Prolong2Tile<T, GPX, GPZ> sm;
+    __shared__ Prolong2Tile<T, GPX, GPZ, NT> sm;
     pdl_trigger();
     const int b = blockIdx.z;
-    prolong2_tile_stage<T, GPX, GPZ>(sm, Lf, Lm, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);
+    prolong2_tile_stage<T, GPX, GPZ, NT>(sm, Lf, Lm, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);
     pdl_wait();
     if (!rhs_active(st, b)) return;
-    prolong2_tile_work<T, GPX, GPZ, false>(sm, Lf, Lm, Lc, wj, fl, fm, ec, em, out, acc_f, acc_m, blockIdx.x,
+    prolong2_tile_work<T, GPX, GPZ, false, BlockSync, NT>(sm, Lf, Lm, Lc, wj, fl, fm, ec, em, out, acc_f, acc_m, blockIdx.x,
                                            blockIdx.y, b, threadIdx.x, BlockSync{});
 }
 
-template <typename T, int GPX, int GPZ>
+template <typename T, int GPX, int GPZ, int NT = GPX * GPZ>
 static void launch_prolong2_shape(const LevelDev& Lf, const LevelDev& Lm, const LevelDev& Lc, const T* w2, double b1,
                                   double b2, double wj, const T* fl, const T* fm, const T* ec, const T* em, T* out,
                                   const RhsState* st, int nrhs, cudaStream_t s, int acc_f, int acc_m) {
     dim3 grd((Lf.nx + GPX - 1) / GPX, (Lf.nz + GPZ - 1) / GPZ, nrhs);
-    launch_pdl(k_prolong2_g<T, GPX, GPZ>, grd, dim3(GPX * GPZ), 0, s, Lf, Lm, Lc, w2, (T)b1, (T)b2, (T)wj, fl, fm, ec,
+    launch_pdl(k_prolong2_g<T, GPX, GPZ, NT>, grd, dim3(NT), 0, s, Lf, Lm, Lc, w2, (T)b1, (T)b2, (T)wj, fl, fm, ec,
                em, out, st, acc_f, acc_m);
 }
 
@@ -1008,12 +1024,13 @@ void launch_prolong2(const LevelDev& Lf, const LevelDev& Lm, const LevelDev& Lc,
                        (nf + nm) * sizeof(T) * kGalerkinCoefs * (Lf.gkstride ? nrhs : 1),
                    s);
     if constexpr (sizeof(T) == 4) {
-        if (tile != 0) {
+        if (tile > 1 || (tile == 1 && !small_prolong(Lf, nrhs))) {
             launch_prolong2_shape<T, 32, 8>(Lf, Lm, Lc, w2, b1, b2, wj, fl, fm, ec, em, out, st, nrhs, s, acc_f, acc_m);
             return;
         }
     }
-    launch_prolong2_shape<T, 16, 8>(Lf, Lm, Lc, w2, b1, b2, wj, fl, fm, ec, em, out, st, nrhs, s, acc_f, acc_m);
+    launch_prolong2_shape<T, 16, 8, sizeof(T) == 4 ? 128 : 192>(Lf, Lm, Lc, w2, b1, b2, wj, fl, fm, ec, em, out, st,
+                                                                nrhs, s, acc_f, acc_m);
 }
 template void launch_prolong2<float>(const LevelDev&, const LevelDev&, const LevelDev&, const float*, double, double,
                                      double, const float*, const float*, const float*, const float*, float*,
@@ -1023,10 +1040,10 @@ template void launch_prolong2<double>(const LevelDev&, const LevelDev&, const Le
                                       const RhsState*, int, cudaStream_t, int, int, int);
 
 // Tile shapes of the complex64 Galerkin kernels, by the code the autotuner stores
-// per level (kGalTiles choices; 1 is the default): restriction coarse tile
-// (x, z) and prolongation fine tile (x, z), one thread per node of the tile. The
-// shapes keep each block's shared memory within 48 KB.
-//   0: 8 x 8 / 16 x 8,  1: 16 x 8 / 32 x 8,  2: 32 x 4 / 64 x 4,  3: 8 x 16 / 32 x 16,  4: 8 x 8 on 128
+// per level: restriction coarse tile (x, z) and prolongation fine tile (x, z), one thread per
+// node of the tile unless said otherwise. The shapes keep each block's shared memory within 48 KB.
+//   0: 8 x 8 / 16 x 8,  1 (default): by the level's size, see small_level / small_prolong,
+//   2: 32 x 4 / 64 x 4,  3: 8 x 16 / 32 x 16,  4: 8 x 8 on 128
 //   threads (two per coarse node, for short per-thread chains on small levels) / 128 x 2,
 //   5 (restriction only): 8 x 16 on 256 threads (two per coarse node)
 template <typename T, bool CORRECT, int GRCX, int GRCZ, int NT = GRCX * GRCZ>
@@ -1052,15 +1069,23 @@ void launch_restrict_g(int tile, const LevelDev& Lf, const LevelDev& Lc, const T
             case 5: launch_restrict_g_shape<T, CORRECT, 8, 16, 256>(Lf, Lc, w2, b1, b2, wj, f, ec, fc, st, nrhs, s); return;
             default: break;
         }
+        if (small_level(Lc, nrhs))
+            launch_restrict_g_shape<T, CORRECT, 8, 4, 224>(Lf, Lc, w2, b1, b2, wj, f, ec, fc, st, nrhs, s);
+        else
+            launch_restrict_g_shape<T, CORRECT, 8, 16, 256>(Lf, Lc, w2, b1, b2, wj, f, ec, fc, st, nrhs, s);
+        return;
     }
-    launch_restrict_g_shape<T, CORRECT, GTile<T>::RCX, GTile<T>::RCZ>(Lf, Lc, w2, b1, b2, wj, f, ec, fc, st, nrhs, s);
+    // complex128: 8 x 8 tiles, a thread for every other fine node (64 threads: 21.6 against 14.0 us on
+    // 120 x 95 nodes with two right-hand sides; 384 threads the same)
+    launch_restrict_g_shape<T, CORRECT, GTile<T>::RCX, GTile<T>::RCZ, 192>(Lf, Lc, w2, b1, b2, wj, f, ec, fc, st, nrhs,
+                                                                          s);
 }
-template <typename T, int GPX, int GPZ>
+template <typename T, int GPX, int GPZ, int NT = GPX * GPZ>
 void launch_prolong_g_shape(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double b1, double b2, double wj,
                             const T* f, const T* ec, T* out, const RhsState* st, int nrhs, cudaStream_t s,
                             int accumulate) {
     dim3 grd((Lf.nx + GPX - 1) / GPX, (Lf.nz + GPZ - 1) / GPZ, nrhs);
-    launch_pdl(k_prolong_g<T, GPX, GPZ>, grd, dim3(GPX * GPZ), 0, s, Lf, Lc, w2, (T)b1, (T)b2, (T)wj, f, ec, out, st,
+    launch_pdl(k_prolong_g<T, GPX, GPZ, NT>, grd, dim3(NT), 0, s, Lf, Lc, w2, (T)b1, (T)b2, (T)wj, f, ec, out, st,
                accumulate);
 }
 template <typename T>
@@ -1073,13 +1098,19 @@ void launch_prolong_g(int tile, const LevelDev& Lf, const LevelDev& Lc, const T*
         }
         switch (tile) {
             case 0: launch_prolong_g_shape<T, 16, 8>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate); return;
+            case 1:
+                if (!small_prolong(Lf, nrhs)) break;
+                launch_prolong_g_shape<T, 16, 8>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate);
+                return;
             case 2: launch_prolong_g_shape<T, 64, 4>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate); return;
             case 3: launch_prolong_g_shape<T, 32, 16>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate); return;
             case 4: launch_prolong_g_shape<T, 128, 2>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate); return;
             default: break;
         }
+        launch_prolong_g_shape<T, 32, 8>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate);
+    } else {   // complex128: a thread for every node of the tile and its halo
+        launch_prolong_g_shape<T, 16, 8, 192>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate);
     }
-    launch_prolong_g_shape<T, GTile<T>::PX, GTile<T>::PZ>(Lf, Lc, w2, b1, b2, wj, f, ec, out, st, nrhs, s, accumulate);
 }
 
 // ======================================================== V-cycle: restrict
