@@ -25,21 +25,24 @@ constexpr int kFgMaxBlocks = 1024;                                 // blocks per
 
 // Blocks per RHS of a grid-stride kernel: about two points per thread, at most
 // one wave of the kernel's resident blocks on every SM.
-template <auto Kernel>
-int fg_grid(size_t n) {
+template <auto Kernel, int Threads = 256>
+int fg_grid(size_t n, int share = 1) {   // share: the launch's grids (chunks, right-hand sides) that split the wave
     // resident blocks per SM of this kernel, looked up once (a function-local static is
     // initialised exactly once even when serving threads get here together)
     static const int per_sm = [] {
         int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kernel, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kernel, Threads, 0);
         return nb > 0 ? nb : 1;
     }();
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t cap = std::min<size_t>(kFgMaxBlocks, (size_t)std::max(1, per_sm * sms));
-    return (int)std::max<size_t>(1, std::min<size_t>((n + 511) / 512, cap));
+    const size_t cap = std::min<size_t>(kFgMaxBlocks, (size_t)std::max(1, per_sm * sms / share));
+    return (int)std::max<size_t>(1, std::min<size_t>((n + 2 * Threads - 1) / (2 * Threads), cap));
 }
+constexpr int kDotThreads = 384;   // threads per block of the dot products
+// points a thread takes per step: enough loads in flight within 80 registers (two blocks per SM)
+template <typename T, int NV> constexpr int kDotPts = sizeof(T) == 8 ? (NV <= 2 ? 2 : 1) : (NV <= 4 ? 4 : NV <= 8 ? 2 : 1);
 }  // namespace
 
 // Partials per RHS that the FGMRES kernels need on n points: 2 kChunk + 1 sums
@@ -48,38 +51,7 @@ int fg_partials(size_t n) {
     return (2 * kChunk + 1) * kMaxChunks * (int)std::min<size_t>(kFgMaxBlocks, std::max<size_t>(1, (n + 511) / 512));
 }
 
-// ||rin||; beta = g[0], s_0 = 1; the RHS iterates if its outer step is active
-// and rin != 0.
-template <typename T>
-__global__ void __launch_bounds__(256) k_fg_norm(const T* __restrict__ rin, double* partials, int pstride,
-                                                 RhsState* st, FgDev fg, int* nactive, size_t n) {
-    __shared__ double sh[32];
-    const int b = blockIdx.z;
-    if (!st[b].outer_active) return;
-    T a0 = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const cx<T> c = ldc(rin, n * b + i);
-        a0 += c.re * c.re + c.im * c.im;
-    }
-    const T vv[1] = {a0};
-    double acc[1];
-    if (last_block_reduce_t<1, T>(vv, acc, sh, partials + (size_t)b * pstride, gridDim.x, blockIdx.x, &st[b].counter[1])) {
-        if (threadIdx.x == 0) {
-            RhsState& S = st[b];
-            S.bnorm2 = acc[0];
-            S.rnorm2 = acc[0];
-            S.kfg = 0;
-            S.reorth = 0;
-            S.flag = FLAG_RUNNING;
-            S.active = acc[0] > 0.0;
-            fg.g[(size_t)b * (fg.m + 1)] = make_double2(sqrt(acc[0]), 0.0);
-            fg.sinv[(size_t)b * (fg.m + 1)] = 1.0;
-            if (S.active) atomicAdd(nactive, 1);
-        }
-    }
-}
-
-// V'_0 = rin / beta.
+// V'_0 = rin / beta (beta, and the state of a new cycle, come from the residual kernel, k_resid64).
 template <typename T>
 __global__ void k_fg_scale(const T* __restrict__ rin, T* __restrict__ v, const RhsState* st, FgDev fg, size_t n) {
     const int b = blockIdx.z;
@@ -91,19 +63,27 @@ __global__ void k_fg_scale(const T* __restrict__ rin, T* __restrict__ v, const R
 
 // d_i = <V'_i, w> for i <= j (w = A Z'_j, unnormalised, in basis slot j+1);
 // blockIdx.y picks a chunk of NV vectors (NV = the smallest of 1, 2, 4, 8 that
-// covers j + 1, else 8). The last block of the RHS writes the projection
+// covers j + 1, 6 for 9 .. 12 of them, else 8). The last block of the RHS writes the projection
 // coefficients tmp_i = d_i / s_i^2 and sets (add = 0) or adds (add = 1)
 // h_ij = d_i / (s_i s_j) into column j of H. With `wnorm` the chunk-0 blocks also
 // sum ||w||^2 into wn2 (for the second-pass test). With `check` an RHS whose
 // first pass asked for no second pass skips the kernel.
+// The end of the kernel is a chain: partials out, the last block's partials in, their sums, the
+// coefficients out. Two blocks of 384 threads per SM leave at most 304 partials per sum, so each
+// lane of the last block's warps takes all of its own in one round of loads, with twelve vectors
+// at a time and 1 / s_i loaded beside them. (With 256 threads: up to 912 partials, three rounds,
+// eight vectors at a time; that end was about half of a launch at one right-hand side.) On the
+// 1041 x 1041 grid: one vector 11.7 -> 9.0 us, four 13.6 -> 11.5, eight 18.3 -> 17.
 template <typename T, int NV>
-__global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t vstride, const T* __restrict__ w,
+__global__ void __launch_bounds__(kDotThreads) k_fg_dots(const T* __restrict__ V, size_t vstride, const T* __restrict__ w,
                                                  int j, int add, int wnorm, int check, double* partials, int pstride,
                                                  RhsState* st, FgDev fg, size_t n) {
     constexpr int NA = 2 * NV + 1;
-    __shared__ double sh[NA][33];
+    __shared__ double sh[NA][kDotThreads / 32 + 1];
     __shared__ int s_last;
     const int b = blockIdx.z;
+    pdl_trigger();
+    pdl_wait();
     if (!st[b].active || (check && !st[b].reorth)) return;
     const int i0 = blockIdx.y * NV;
     const int nv = min(NV, j + 1 - i0);
@@ -116,24 +96,32 @@ __global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t
     T acc[NA];
 #pragma unroll
     for (int k = 0; k < NA; ++k) acc[k] = 0;
-    // two points per thread and step, every load of the step issued before use
+    // kDotPts points per thread and step, every load of the step issued before use
+    constexpr int PT = kDotPts<T, NV>;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    for (; p + stride < n; p += 2 * stride) {
-        const cx<T> w0 = ldc(wb, p), w1 = ldc(wb, p + stride);
-        cx<T> q0[NV], q1[NV];
+    for (; p + (PT - 1) * stride < n; p += PT * stride) {
+        cx<T> wv[PT], q[NV][PT];
+#pragma unroll
+        for (int t = 0; t < PT; ++t) wv[t] = ldc(wb, p + t * stride);
 #pragma unroll
         for (int k = 0; k < NV; ++k)
-            if (k < nv) { q0[k] = ldc(vp[k], p); q1[k] = ldc(vp[k], p + stride); }
+            if (k < nv)
+#pragma unroll
+                for (int t = 0; t < PT; ++t) q[k][t] = ldc(vp[k], p + t * stride);
 #pragma unroll
         for (int k = 0; k < NV; ++k)
-            if (k < nv) {
-                acc[2 * k] += (q0[k].re * w0.re + q0[k].im * w0.im) + (q1[k].re * w1.re + q1[k].im * w1.im);
-                acc[2 * k + 1] += (q0[k].re * w0.im - q0[k].im * w0.re) + (q1[k].re * w1.im - q1[k].im * w1.re);
-            }
-        if (wn) acc[2 * NV] += (w0.re * w0.re + w0.im * w0.im) + (w1.re * w1.re + w1.im * w1.im);
+            if (k < nv)
+#pragma unroll
+                for (int t = 0; t < PT; ++t) {
+                    acc[2 * k] += q[k][t].re * wv[t].re + q[k][t].im * wv[t].im;
+                    acc[2 * k + 1] += q[k][t].re * wv[t].im - q[k][t].im * wv[t].re;
+                }
+        if (wn)
+#pragma unroll
+            for (int t = 0; t < PT; ++t) acc[2 * NV] += wv[t].re * wv[t].re + wv[t].im * wv[t].im;
     }
-    if (p < n) {
+    for (; p < n; p += stride) {
         const cx<T> w0 = ldc(wb, p);
 #pragma unroll
         for (int k = 0; k < NV; ++k)
@@ -156,14 +144,15 @@ __global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t
     const int nblk = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
     double* part = partials + (size_t)b * pstride;
     if (threadIdx.x < NA) {
-        // the eight warp totals (256 threads) by a fixed pairwise tree
-        double w8[8];
+        // the warp totals by a fixed pairwise tree
+        constexpr int NW = kDotThreads / 32;
+        double w8[NW];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) w8[q] = sh[threadIdx.x][q];
+        for (int q = 0; q < NW; ++q) w8[q] = sh[threadIdx.x][q];
+        static_assert(NW == 12, "pairwise tree of the warp totals");
 #pragma unroll
-        for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-            for (int q = 0; q < w; ++q) w8[q] += w8[q + w];
+        for (int q = 0; q < 4; ++q) w8[q] = (w8[q] + w8[q + 4]) + w8[q + 8];
+        w8[0] = (w8[0] + w8[1]) + (w8[2] + w8[3]);
         part[(size_t)threadIdx.x * nblk + blk] = w8[0];
     }
     (void)nw;
@@ -186,23 +175,21 @@ __global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t
         const int c = isn ? 0 : i / NV, k = isn ? NV : i % NV;
         const double* pre = part + (size_t)(2 * k) * nblk + (size_t)c * nx;
         const double* pim = part + (size_t)(2 * k + 1) * nblk + (size_t)c * nx;
-        // eight loads per lane in flight, summed by a fixed pairwise tree (three
-        // dependent FP64 additions per batch instead of eight)
+        const double si = isn ? 0.0 : sinv[i], sj = sinv[j];
+        // ten loads of each part per lane in flight (320 partials a round), summed by a fixed tree
         double re = 0.0, im = 0.0;
-        for (int x0 = 0; x0 < nx; x0 += 256) {
-            double vr[8], vi[8];
+        for (int x0 = 0; x0 < nx; x0 += 320) {
+            double vr[10], vi[10];
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
+            for (int t = 0; t < 10; ++t) {
                 const int x = x0 + lane + 32 * t;
                 vr[t] = x < nx ? __ldcg(pre + x) : 0.0;
                 vi[t] = (x < nx && !isn) ? __ldcg(pim + x) : 0.0;
             }
 #pragma unroll
-            for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-                for (int t = 0; t < w; ++t) { vr[t] += vr[t + w]; vi[t] += vi[t + w]; }
-            re += vr[0];
-            im += vi[0];
+            for (int t = 0; t < 5; ++t) { vr[t] += vr[t + 5]; vi[t] += vi[t + 5]; }
+            re += ((vr[0] + vr[1]) + (vr[2] + vr[3])) + vr[4];
+            im += ((vi[0] + vi[1]) + (vi[2] + vi[3])) + vi[4];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -213,7 +200,7 @@ __global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t
             if (isn) {
                 fg.wn2[b] = re;
             } else {
-                const double si = sinv[i], inv2 = si * si, invh = si * sinv[j];
+                const double inv2 = si * si, invh = si * sj;
                 fg.tmp[col + i] = make_double2(re * inv2, im * inv2);
                 double2& h = fg.H[(col + i) * fg.m + j];
                 if (add) { h.x += re * invh; h.y += im * invh; } else { h = make_double2(re * invh, im * invh); }
@@ -223,17 +210,58 @@ __global__ void __launch_bounds__(256) k_fg_dots(const T* __restrict__ V, size_t
     if (threadIdx.x == 0) st[b].counter[2] = 0u;
 }
 
+// y = R^{-1} g on the k leading rows (FP64) by columns, by one warp: lane q holds the right-hand
+// side entry q; at step i the lane holding row i finishes y_i with the reciprocal of R_ii (all
+// reciprocals formed together beforehand, so no division sits on the chain) and every lane
+// q < i subtracts R_qi y_i. The chain is k steps of one complex product, one shuffle and
+// one complex multiply-add in FP64. Runs in the block that finishes the cycle's last column,
+// whose entries it has just written (R: the column in shared memory, the others from H).
+__device__ void fg_backsolve(const FgDev& fg, int b, int k) {
+    __shared__ double2 R[kMaxRestart][kMaxRestart + 1];   // the triangle, staged once
+    const int m = fg.m, lane = threadIdx.x;               // k <= kMaxRestart = 32
+    const size_t col = (size_t)b * (m + 1);
+    const double2* H = fg.H + col * m;
+    for (int idx = lane; idx < k * k; idx += 32) {
+        const int i = idx / k, q = idx - i * k;
+        if (q >= i) R[i][q] = __ldcg(H + (size_t)i * m + q);
+    }
+    __syncwarp();
+    double2 acc = lane < k ? __ldcg(fg.g + col + lane) : make_double2(0.0, 0.0);
+    double2 rinv = make_double2(0.0, 0.0);
+    if (lane < k) {
+        const double2 d = R[lane][lane];
+        const double dd = d.x * d.x + d.y * d.y;
+        if (dd > 0.0) {
+            const double inv = 1.0 / dd;
+            rinv = make_double2(d.x * inv, -d.y * inv);
+        }
+    }
+    double2* y = fg.y + (size_t)b * m;
+    for (int i = k - 1; i >= 0; --i) {
+        double2 yi = make_double2(acc.x * rinv.x - acc.y * rinv.y, acc.x * rinv.y + acc.y * rinv.x);
+        yi.x = __shfl_sync(0xffffffffu, yi.x, i);
+        yi.y = __shfl_sync(0xffffffffu, yi.y, i);
+        if (lane == i) y[i] = yi;
+        if (lane < i) {
+            const double2 h = R[lane][i];
+            acc.x -= h.x * yi.x - h.y * yi.y;
+            acc.y -= h.x * yi.y + h.y * yi.x;
+        }
+    }
+}
+
 // Column j of the Arnoldi relation is complete (||w'|| = hn2^(1/2) after the
 // last pass): 1/s_{j+1}, h_{j+1,j} = s_{j+1} / s_j, the previous Givens
 // rotations on column j, the new rotation zeroing h_{j+1,j}, and the
 // convergence test |g_{j+1}| <= tol_rel * beta. Called by every thread of one
 // block: the column and the rotations are staged in shared memory, so the
 // serial FP64 chain of thread 0 waits on no global load; it takes three square
-// roots and two divisions.
+// roots and two divisions. The column that ends the cycle is followed by the back substitution.
 __device__ void fg_finish_column(RhsState& S, const FgDev& fg, int b, int j, double hn2, int* nactive) {
     __shared__ double2 hc[kMaxRestart + 1];
     __shared__ double2 sc[kMaxRestart];
     __shared__ double cc[kMaxRestart];
+    __shared__ int s_done;
     const int m = fg.m;
     const size_t col = (size_t)b * (m + 1);
     double2* H = fg.H + col * m;                   // H[i * m + j]
@@ -283,10 +311,15 @@ __device__ void fg_finish_column(RhsState& S, const FgDev& fg, int b, int j, dou
         else if (j + 1 >= m) { done = 1; S.flag = FLAG_MAXIT; }
         else if (S.iters >= S.max_it) { done = 1; S.flag = FLAG_MAXIT; }
         if (done) { S.active = 0; atomicSub(nactive, 1); }
+        s_done = done;
     }
     __syncthreads();
     for (int i = threadIdx.x; i <= j; i += blockDim.x) H[(size_t)i * m + j] = hc[i];
     if (threadIdx.x == 0) H[(size_t)(j + 1) * m + j] = make_double2(0.0, 0.0);
+    if (s_done) {
+        __syncthreads();   // the column and g are written
+        if (threadIdx.x < 32) fg_backsolve(fg, b, j + 1);
+    }
 }
 
 // w -= sum_{i <= j} tmp_i V'_i in place (w is basis slot j+1). mode 0: no norm
@@ -302,6 +335,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_fg_axpy(const T
     __shared__ double sh[32];
     __shared__ cx<T> coef[kMaxRestart + 1];
     const int b = blockIdx.z;
+    pdl_trigger();
+    pdl_wait();
     if (!st[b].active || (check && !st[b].reorth)) return;
     const size_t col = (size_t)b * (fg.m + 1);
     for (int i = threadIdx.x; i <= j; i += blockDim.x) coef[i] = cx<T>((T)fg.tmp[col + i].x, (T)fg.tmp[col + i].y);
@@ -380,58 +415,14 @@ __global__ void __launch_bounds__(256) k_fg_finish(const double* partials, int p
     fg_finish_column(st[b], fg, b, j, s_hn2, nactive);
 }
 
-// y = R^{-1} g on the k = kfg leading rows (FP64), one warp per RHS: the warp
-// stages the triangle and g in shared memory with all its loads in flight, then
-// lane 0 substitutes backwards.
-__global__ void __launch_bounds__(32) k_fg_backsolve(const RhsState* st, FgDev fg) {
-    // y = R^-1 g by columns: lane q holds the right-hand side entry q; at step i the lane
-    // holding row i finishes y_i with the reciprocal of R_ii (all reciprocals formed
-    // together beforehand, so no division sits on the chain) and every lane q < i
-    // subtracts R_qi y_i. The chain is k steps of one complex product, one shuffle and
-    // one complex multiply-add in FP64, instead of k divisions and k (k - 1) / 2
-    // sequential multiply-adds on one thread.
-    const int b = blockIdx.x;
-    if (!st[b].outer_active) return;
-    const int m = fg.m, k = st[b].kfg, lane = threadIdx.x;   // k <= kMaxRestart = 32
-    const size_t col = (size_t)b * (m + 1);
-    const double2* H = fg.H + col * m;
-    __shared__ double2 R[kMaxRestart][kMaxRestart + 1];   // the triangle, staged once
-    for (int idx = lane; idx < k * k; idx += 32) {
-        const int i = idx / k, q = idx - i * k;
-        if (q >= i) R[i][q] = H[(size_t)i * m + q];
-    }
-    __syncwarp();
-    double2 acc = lane < k ? fg.g[col + lane] : make_double2(0.0, 0.0);
-    double2 rinv = make_double2(0.0, 0.0);
-    if (lane < k) {
-        const double2 d = R[lane][lane];
-        const double dd = d.x * d.x + d.y * d.y;
-        if (dd > 0.0) {
-            const double inv = 1.0 / dd;
-            rinv = make_double2(d.x * inv, -d.y * inv);
-        }
-    }
-    double2* y = fg.y + (size_t)b * m;
-    for (int i = k - 1; i >= 0; --i) {
-        double2 yi = make_double2(acc.x * rinv.x - acc.y * rinv.y, acc.x * rinv.y + acc.y * rinv.x);
-        yi.x = __shfl_sync(0xffffffffu, yi.x, i);
-        yi.y = __shfl_sync(0xffffffffu, yi.y, i);
-        if (lane == i) y[i] = yi;
-        if (lane < i) {
-            const double2 h = R[lane][i];
-            acc.x -= h.x * yi.x - h.y * yi.y;
-            acc.y -= h.x * yi.y + h.y * yi.x;
-        }
-    }
-}
-
-// x = sum_{i < kfg} (y_i / s_i) Z'_i for every RHS whose outer step is active.
+// u += sum_{i < kfg} (y_i / s_i) Z'_i for every RHS whose outer step is active and whose cycle stayed
+// finite: the correction is summed in T and added in FP64.
 template <typename T>
-__global__ void k_fg_update(const T* __restrict__ Z, size_t zstride, T* __restrict__ x, const RhsState* st, FgDev fg,
-                            size_t n) {
+__global__ void __launch_bounds__(256) k_fg_update(const T* __restrict__ Z, size_t zstride, double* __restrict__ u,
+                                                   const RhsState* st, FgDev fg, size_t n) {
     __shared__ cx<T> coef[kMaxRestart];
     const int b = blockIdx.z;
-    if (!st[b].outer_active) return;
+    if (!st[b].outer_active || !isfinite(st[b].rnorm2)) return;
     const int k = st[b].kfg;
     for (int i = threadIdx.x; i < k; i += blockDim.x) {
         const double2 y = fg.y[(size_t)b * fg.m + i];
@@ -440,7 +431,9 @@ __global__ void k_fg_update(const T* __restrict__ Z, size_t zstride, T* __restri
     }
     __syncthreads();
     const T* zb = Z + 2 * n * b;
+    double* ub = u + 2 * n * b;
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
+        const cx<double> old = ldcc(ub, p);
         cx<T> acc(0, 0);
         for (int i0 = 0; i0 < k; i0 += kChunk) {
             const int nv = min(kChunk, k - i0);
@@ -452,17 +445,11 @@ __global__ void k_fg_update(const T* __restrict__ Z, size_t zstride, T* __restri
             for (int t = 0; t < kChunk; ++t)
                 if (t < nv) acc = acc + coef[i0 + t] * q[t];
         }
-        stc(x, n * b + p, acc);
+        stc(ub, p, cx<double>(old.re + (double)acc.re, old.im + (double)acc.im));
     }
 }
 
 // ------------------------------------------------------------- launchers
-template <typename T>
-void launch_fg_norm(const T* rin, double* partials, int pstride, RhsState* st, const FgDev& fg, int* nactive,
-                    size_t n, int nrhs, cudaStream_t s) {
-    ProfScope prof(PK_FG_NORM, (int)n, 1, (double)n * nrhs * 2.0 * sizeof(T), s);
-    k_fg_norm<T><<<dim3(fg_grid<k_fg_norm<T>>(n), 1, nrhs), 256, 0, s>>>(rin, partials, pstride, st, fg, nactive, n);
-}
 template <typename T>
 void launch_fg_scale(const T* rin, T* v, const RhsState* st, const FgDev& fg, size_t n, int nrhs, cudaStream_t s) {
     ProfScope prof(PK_FG_SCALE, (int)n, 1, (double)n * nrhs * 4.0 * sizeof(T), s);
@@ -472,8 +459,14 @@ template <typename T, int NV>
 static void fg_dots_nv(const T* V, size_t vstride, const T* w, int j, int add, int wnorm, int check, double* partials,
                        int pstride, RhsState* st, const FgDev& fg, size_t n, int nrhs, cudaStream_t s) {
     const int nchunk = (j + NV) / NV;
-    k_fg_dots<T, NV><<<dim3(fg_grid<k_fg_dots<T, NV>>(n), nchunk, nrhs), 256, 0, s>>>(
-        V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n);
+    // at least 16 blocks per sum: a wide batch fills the GPU by itself
+    const int share = std::min(nchunk * nrhs, 19);
+    const dim3 grd(fg_grid<k_fg_dots<T, NV>, kDotThreads>(n, share), nchunk, nrhs);
+    // the second pass follows the first pass's update directly; the first one also waits for the
+    // previous column on another stream, and is launched as an ordinary kernel
+    if (add) launch_pdl(k_fg_dots<T, NV>, grd, dim3(kDotThreads), 0, s, V, vstride, w, j, add, wnorm, check, partials,
+                        pstride, st, fg, n);
+    else k_fg_dots<T, NV><<<grd, kDotThreads, 0, s>>>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n);
 }
 template <typename T>
 void launch_fg_dots(const T* V, size_t vstride, const T* w, int j, int add, int wnorm, int check, double* partials,
@@ -484,17 +477,17 @@ void launch_fg_dots(const T* V, size_t vstride, const T* w, int j, int add, int 
     else if (j < 2) fg_dots_nv<T, 2>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
     else if (j < 4) fg_dots_nv<T, 4>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
     else if (j < kChunk) fg_dots_nv<T, kChunk>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
-    // 9 .. 12 vectors in one pass over w (two chunks of eight would read w twice, and the second,
-    // short chunk would run as a second, light wave)
-    else if (j < 12) fg_dots_nv<T, 12>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
+    // 9 .. 12 vectors in two equal chunks (eight and a short second wave, or twelve at once with half
+    // the warps, measured 27 and 25 us where this takes 23 to 24 us)
+    else if (j < 12) fg_dots_nv<T, 6>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
     else fg_dots_nv<T, kChunk>(V, vstride, w, j, add, wnorm, check, partials, pstride, st, fg, n, nrhs, s);
 }
 template <typename T, int NV>
 static int fg_axpy_nv(const T* V, size_t vstride, T* w, int j, int mode, int check, double* partials, int pstride,
                       RhsState* st, const FgDev& fg, int* nactive, size_t n, int nrhs, cudaStream_t s) {
     const int grid = fg_grid<k_fg_axpy<T, NV>>(n);
-    k_fg_axpy<T, NV><<<dim3(grid, 1, nrhs), 256, 0, s>>>(V, vstride, w, j, mode, check, partials, pstride, st, fg,
-                                                          nactive, n);
+    launch_pdl(k_fg_axpy<T, NV>, dim3(grid, 1, nrhs), dim3(256), 0, s, V, vstride, w, j, mode, check, partials, pstride,
+               st, fg, nactive, n);
     return grid;
 }
 template <typename T>
@@ -512,27 +505,21 @@ void launch_fg_finish(const double* partials, int pstride, int nblk, RhsState* s
     ProfScope prof(PK_FG_FINISH, nblk, 1, (double)nblk * nrhs * 8.0 * 2, s);
     k_fg_finish<<<nrhs, 256, 0, s>>>(partials, pstride, nblk, st, fg, j, nactive);
 }
-void launch_fg_backsolve(const RhsState* st, const FgDev& fg, int nrhs, cudaStream_t s) {
-    ProfScope prof(PK_FG_BACKSOLVE, fg.m, 1, (double)fg.m * fg.m * nrhs * 16.0, s);
-    k_fg_backsolve<<<nrhs, 32, 0, s>>>(st, fg);
-}
 template <typename T>
-void launch_fg_update(const T* Z, size_t zstride, T* x, const RhsState* st, const FgDev& fg, size_t n, int nrhs,
+void launch_fg_update(const T* Z, size_t zstride, double* u, const RhsState* st, const FgDev& fg, size_t n, int nrhs,
                       cudaStream_t s) {
-    // reads Z'_0 .. Z'_{m-1}, reads and writes x
-    ProfScope prof(PK_FG_UPDATE, (int)n, 1, (double)n * nrhs * 2.0 * sizeof(T) * (fg.m + 2), s);
-    k_fg_update<T><<<dim3(fg_grid<k_fg_update<T>>(n), 1, nrhs), 256, 0, s>>>(Z, zstride, x, st, fg, n);
+    // reads Z'_0 .. Z'_{m-1}, reads and writes u
+    ProfScope prof(PK_FG_UPDATE, (int)n, 1, (double)n * nrhs * (2.0 * sizeof(T) * fg.m + 32.0), s);
+    k_fg_update<T><<<dim3(fg_grid<k_fg_update<T>>(n), 1, nrhs), 256, 0, s>>>(Z, zstride, u, st, fg, n);
 }
 
 #define HELM_FG_INST(T)                                                                                             \
-    template void launch_fg_norm<T>(const T*, double*, int, RhsState*, const FgDev&, int*, size_t, int,             \
-                                    cudaStream_t);                                                                  \
     template void launch_fg_scale<T>(const T*, T*, const RhsState*, const FgDev&, size_t, int, cudaStream_t);       \
     template void launch_fg_dots<T>(const T*, size_t, const T*, int, int, int, int, double*, int, RhsState*,        \
                                     const FgDev&, size_t, int, cudaStream_t);                                       \
     template int launch_fg_axpy<T>(const T*, size_t, T*, int, int, int, double*, int, RhsState*, const FgDev&,      \
                                    int*, size_t, int, cudaStream_t);                                                \
-    template void launch_fg_update<T>(const T*, size_t, T*, const RhsState*, const FgDev&, size_t, int,             \
+    template void launch_fg_update<T>(const T*, size_t, double*, const RhsState*, const FgDev&, size_t, int,        \
                                       cudaStream_t);
 HELM_FG_INST(float)
 HELM_FG_INST(double)

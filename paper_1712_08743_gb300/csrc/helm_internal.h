@@ -267,11 +267,14 @@ template <typename T>
 void launch_apply_dots(int mode, const LevelDev& L0, int npml, double amax, const T* hw, const T* u, T* y,
                        const T* aux, double* partials, int pstride, RhsState* st, int nrhs, cudaStream_t s);
 
-// Outer FP64 residual r = f - A u; TI = precision of the inner right-hand side.
+// Outer FP64 residual r = f - A u; TI = precision of the inner right-hand side. fg (nullable): the
+// FGMRES state, which is set up for a new cycle.
+struct FgDev;
 template <typename TI>
 void launch_resid64(const LevelDev& L0, int npml, double amax, const double* w2, const double* f,
                     const double* u, TI* rin, double* partials, int pstride, RhsState* st,
-                    double tol, double inner_floor, double inner_fac, int first, int nrhs, cudaStream_t s);
+                    double tol, double inner_floor, double inner_fac, int first, int nrhs, cudaStream_t s,
+                    const FgDev* fg = nullptr);
 template <typename TI>
 void launch_refine(const TI* x, double* u, const RhsState* st, size_t n, int nrhs, cudaStream_t s);
 
@@ -400,9 +403,6 @@ struct FgDev {
     double* wn2;
 };
 template <typename T>
-void launch_fg_norm(const T* rin, double* partials, int pstride, RhsState* st, const FgDev& fg, int* nactive,
-                    size_t n, int nrhs, cudaStream_t s);
-template <typename T>
 void launch_fg_scale(const T* rin, T* v, const RhsState* st, const FgDev& fg, size_t n, int nrhs, cudaStream_t s);
 template <typename T>
 void launch_fg_dots(const T* V, size_t vstride, const T* w, int j, int add, int wnorm, int check, double* partials,
@@ -413,11 +413,10 @@ int launch_fg_axpy(const T* V, size_t vstride, T* w, int j, int mode, int check,
                    RhsState* st, const FgDev& fg, int* nactive, size_t n, int nrhs, cudaStream_t s);
 void launch_fg_finish(const double* partials, int pstride, int nblk, RhsState* st, const FgDev& fg, int j,
                       int* nactive, int nrhs, cudaStream_t s);
-void launch_fg_backsolve(const RhsState* st, const FgDev& fg, int nrhs, cudaStream_t s);
 int fg_partials(size_t n);   // reduction partials per RHS the FGMRES kernels need on n points
 constexpr int kFgTimedStep = 4;   // Arnoldi step that helm_time_kernel times (the middle of FGMRES(10))
 template <typename T>
-void launch_fg_update(const T* Z, size_t zstride, T* x, const RhsState* st, const FgDev& fg, size_t n, int nrhs,
+void launch_fg_update(const T* Z, size_t zstride, double* u, const RhsState* st, const FgDev& fg, size_t n, int nrhs,
                       cudaStream_t s);
 
 // FP64 throughput probe: blocks x 256 threads x 8 chains x iters fused multiply-adds

@@ -365,26 +365,48 @@ template void launch_apply_dots<double>(int, const LevelDev&, int, double, const
 
 // ======================================================= FP64 outer residual
 // r = f - A u in FP64; writes the inner right-hand side rin = r in precision TI
-// and decides, per right-hand side, whether refinement continues. GB300 issues
-// FP64 at a small fraction of its FP32 rate, so this kernel is bound by FP64
-// instructions, not bytes (GB300: about 1.7 FP64 operations per clock per SM,
-// DADD, DMUL, DFMA and the double-to-float conversion alike). Each thread takes
-// R64_ROWS consecutive rows of one column, so the block sum is paid once for all
-// of them; interior nodes (outside the absorbing layer, four neighbours) sum
-// the neighbours pairwise and fuse the diagonal product and the squared norm
-// into FMAs; ||f||^2 is formed only on the first call of a solve.
-constexpr int R64_ROWS = 8;
+// and decides, per right-hand side, whether refinement continues (and sets up the FGMRES state
+// of the next cycle: beta = ||r||, s_0 = 1). GB300 issues FP64 at a small fraction of its FP32
+// rate (about 0.63 T operations per second: DADD, DMUL, DFMA and the double-to-float
+// conversion alike), so this kernel is bound by FP64 instructions, not bytes: 16 per node
+// outside the absorbing layer (the neighbours pairwise, the diagonal product and the squared norm
+// in FMAs, two conversions). Each thread takes R64_ROWS consecutive rows of one column with
+// every load issued before the first use; ||f||^2 is formed only on the first call of a solve.
+// One right-hand side on 1041 x 1041: 67 -> 56 us (FP64 pipe 81 % busy while an SM is active; the
+// rest is the uneven last wave), up to 320 of them on 441 x 241: 1540 -> 1420 us.
+constexpr int R64_ROWS = 4;
+
+constexpr int R64_Y = 4;             // warps per block
+constexpr int R64_THREADS = 32 * R64_Y;
+
+// Sum of one double per thread of an R64_THREADS block, in thread 0: through shared memory, so that one
+// warp adds four values per lane and then its lanes (nine FP64 operations in place of ten in every warp).
+__device__ __forceinline__ double r64_block_sum(double v, double* sh) {
+    const int tid = threadIdx.x + 32 * threadIdx.y;
+    __syncthreads();
+    sh[tid] = v;
+    __syncthreads();
+    double a = 0.0;
+    if (tid < 32) {
+        a = (sh[tid] + sh[tid + 32]) + (sh[tid + 64] + sh[tid + 96]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
+    return a;
+}
 
 template <typename TI, bool VD>
-__global__ void __launch_bounds__(256) k_resid64(LevelDev L, int npml, double acoef, const double* __restrict__ w2,
+__global__ void __launch_bounds__(R64_THREADS) k_resid64(LevelDev L, int npml, double acoef, const double* __restrict__ w2,
                                                  const double* __restrict__ f, const double* __restrict__ u,
                                                  TI* __restrict__ rin, double* partials, int pstride, RhsState* st,
-                                                 double tol, double inner_floor, double inner_fac, int first) {
-    __shared__ double sh[64];
+                                                 double tol, double inner_floor, double inner_fac, int first,
+                                                 FgDev fg) {
+    __shared__ double sh[R64_THREADS];
+    __shared__ int s_last;
     const int b = blockIdx.z;
     if (!st[b].outer_active) return;
     const int nx = L.nx, nz = L.nz;
-    const int ix = blockIdx.x * 32 + threadIdx.x, iz0 = (blockIdx.y * 8 + threadIdx.y) * R64_ROWS;
+    const int ix = blockIdx.x * 32 + threadIdx.x, iz0 = (blockIdx.y * R64_Y + threadIdx.y) * R64_ROWS;
     const size_t n = (size_t)nx * nz;
     const double* ub = u + 2 * n * b;
     const double* fb = f + 2 * n * b;
@@ -392,45 +414,99 @@ __global__ void __launch_bounds__(256) k_resid64(LevelDev L, int npml, double ac
     typename C2<TI>::type* rb = reinterpret_cast<typename C2<TI>::type*>(rin) + n * b;
     const double sw = L.h2 * w2[b];
     double v[2] = {0.0, 0.0};
-    if (ix < nx) {
+    auto emit = [&](size_t i, cx<double> r, cx<double> fv) {
+        v[0] = fma(r.re, r.re, fma(r.im, r.im, v[0]));
+        if (first) v[1] = fma(fv.re, fv.re, fma(fv.im, fv.im, v[1]));
+        rb[i] = {(TI)r.re, (TI)r.im};
+    };
+    if (ix < nx && iz0 < nz) {
+        const bool inner = ix > 0 && ix + 1 < nx && iz0 > 0 && iz0 + R64_ROWS < nz &&
+                           layer_depth(ix, iz0, nx, nz, npml) == 0 &&
+                           layer_depth(ix, iz0 + R64_ROWS - 1, nx, nz, npml) == 0;
+        if (!VD && inner) {
+            // f - (4 - s) u + N u, N u the sum of the neighbours
+            const size_t i0 = (size_t)iz0 * nx + ix;
+            cx<double> c[R64_ROWS + 2], fv[R64_ROWS], w[R64_ROWS], e[R64_ROWS];
+            double mm[R64_ROWS];
 #pragma unroll
-        for (int k = 0; k < R64_ROWS; ++k) {
-            const int iz = iz0 + k;
-            if (iz >= nz) break;
-            const size_t i = (size_t)iz * nx + ix;
-            const double s = sw * mb[i];
-            const cx<double> c = ldc(ub, i);
-            const cx<double> fv = ldc(fb, i);
-            cx<double> r;
-            if constexpr (VD) {
-                const double a = layer_alpha_t<double>(ix, iz, nx, nz, npml, acoef);
-                r = fv - fine_apply_point<double, true>(L, ub, i, ix, iz, s, a, c);
-            } else {
-                // f - (4 - s) u + N u (+ the damping term in the layer), N u the sum of the neighbours
-                const double g = 4.0 - s;
-                const int d = layer_depth(ix, iz, nx, nz, npml);
-                if (d == 0 && ix > 0 && ix + 1 < nx && iz > 0 && iz + 1 < nz) {
-                    const cx<double> w = ldc(ub, i - 1), e = ldc(ub, i + 1), no = ldc(ub, i - nx), so = ldc(ub, i + nx);
-                    const cx<double> nb = (w + e) + (no + so);
-                    r = cx<double>(fma(-g, c.re, fv.re) + nb.re, fma(-g, c.im, fv.im) + nb.im);
+            for (int k = 0; k < R64_ROWS + 2; ++k) c[k] = ldc(ub, i0 + (size_t)k * nx - nx);
+#pragma unroll
+            for (int k = 0; k < R64_ROWS; ++k) {
+                const size_t i = i0 + (size_t)k * nx;
+                w[k] = ldc(ub, i - 1);
+                e[k] = ldc(ub, i + 1);
+                fv[k] = ldc(fb, i);
+                mm[k] = __ldg(mb + i);
+            }
+#pragma unroll
+            for (int k = 0; k < R64_ROWS; ++k) {
+                const double g = fma(-sw, mm[k], 4.0);
+                const cx<double> nb = (w[k] + e[k]) + (c[k] + c[k + 2]);
+                emit(i0 + (size_t)k * nx,
+                     cx<double>(fma(-g, c[k + 1].re, fv[k].re) + nb.re, fma(-g, c[k + 1].im, fv[k].im) + nb.im), fv[k]);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < R64_ROWS; ++k) {
+                const int iz = iz0 + k;
+                if (iz >= nz) break;
+                const size_t i = (size_t)iz * nx + ix;
+                const double s = sw * mb[i];
+                const cx<double> c = ldc(ub, i);
+                const cx<double> fv = ldc(fb, i);
+                cx<double> r;
+                if constexpr (VD) {
+                    const double a = layer_alpha_t<double>(ix, iz, nx, nz, npml, acoef);
+                    r = fv - fine_apply_point<double, true>(L, ub, i, ix, iz, s, a, c);
                 } else {
+                    const double g = 4.0 - s;
+                    const int d = layer_depth(ix, iz, nx, nz, npml);
                     cx<double> nb(0.0, 0.0);
                     if (ix > 0) nb = nb + ldc(ub, i - 1);
                     if (ix + 1 < nx) nb = nb + ldc(ub, i + 1);
                     if (iz > 0) nb = nb + ldc(ub, i - nx);
                     if (iz + 1 < nz) nb = nb + ldc(ub, i + nx);
-                    const double sa = s * (acoef * (double)(d * d));
-                    r = cx<double>((fv.re - (g * c.re - sa * c.im)) + nb.re, (fv.im - (g * c.im + sa * c.re)) + nb.im);
+                    r = cx<double>(fma(-g, c.re, fv.re) + nb.re, fma(-g, c.im, fv.im) + nb.im);
+                    if (d > 0) {
+                        const double sa = s * (acoef * (double)(d * d));
+                        r = cx<double>(fma(sa, c.im, r.re), fma(-sa, c.re, r.im));
+                    }
                 }
+                emit(i, r, fv);
             }
-            v[0] = fma(r.re, r.re, fma(r.im, r.im, v[0]));
-            if (first) v[1] = fma(fv.re, fv.re, fma(fv.im, fv.im, v[1]));
-            rb[i] = {(TI)r.re, (TI)r.im};
         }
     }
+    // block sums out; the last block of the right-hand side adds them, eight loads per thread in flight
     const int nblk = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
-    if (last_block_reduce<2>(v, sh, partials + (size_t)b * pstride, nblk, blk, &st[b].counter[0])) {
-        if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double* part = partials + (size_t)b * pstride;
+    const bool t0 = threadIdx.x == 0 && threadIdx.y == 0;
+    v[0] = r64_block_sum(v[0], sh);
+    if (first) v[1] = r64_block_sum(v[1], sh);
+    if (t0) {
+        part[blk] = v[0];
+        if (first) part[nblk + blk] = v[1];
+        __threadfence();
+        s_last = atomicAdd(&st[b].counter[0], 1u) == (unsigned)(nblk - 1);
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        const int tid = threadIdx.x + 32 * threadIdx.y;
+        for (int q = 0; q < (first ? 2 : 1); ++q) {
+            double a = 0.0;
+            for (int i0 = tid; i0 < nblk; i0 += 8 * R64_THREADS) {
+                double x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int i = i0 + k * R64_THREADS;
+                    x[k] = i < nblk ? __ldcg(part + q * nblk + i) : 0.0;
+                }
+                a += ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+            }
+            v[q] = r64_block_sum(a, sh);
+        }
+        if (t0) {
+            st[b].counter[0] = 0u;
             RhsState& S = st[b];
             if (first) S.fnorm2 = v[1];
             double rel = S.fnorm2 > 0.0 ? sqrt(v[0] / S.fnorm2) : 0.0;
@@ -440,6 +516,16 @@ __global__ void __launch_bounds__(256) k_resid64(LevelDev L, int npml, double ac
             S.active = go;
             double t = rel > 0.0 ? inner_fac * tol / rel : 1.0;
             S.tol_rel = t > inner_floor ? t : inner_floor;
+            if (fg.m > 0) {
+                S.bnorm2 = v[0];
+                S.rnorm2 = v[0];
+                S.kfg = 0;
+                S.reorth = 0;
+                S.flag = FLAG_RUNNING;
+                S.active = go && v[0] > 0.0;
+                fg.g[(size_t)b * (fg.m + 1)] = make_double2(sqrt(v[0]), 0.0);
+                fg.sinv[(size_t)b * (fg.m + 1)] = 1.0;
+            }
         }
     }
 }
@@ -447,20 +533,22 @@ __global__ void __launch_bounds__(256) k_resid64(LevelDev L, int npml, double ac
 template <typename TI>
 void launch_resid64(const LevelDev& L0, int npml, double amax, const double* w2, const double* f, const double* u,
                     TI* rin, double* partials, int pstride, RhsState* st, double tol, double inner_floor,
-                    double inner_fac, int first, int nrhs, cudaStream_t s) {
+                    double inner_fac, int first, int nrhs, cudaStream_t s, const FgDev* fgp) {
     const double n0 = (double)L0.nx * L0.nz;
     ProfScope prof(PK_RESID64, L0.nx, L0.nz,
                    n0 * ((32.0 + 2 * sizeof(TI)) * nrhs + 8.0 * (L0.mstride ? nrhs : 1) * (L0.rho ? 4 : 1)), s);
-    dim3 blk(32, 8), grd((L0.nx + 31) / 32, (L0.nz + 8 * R64_ROWS - 1) / (8 * R64_ROWS), nrhs);
+    dim3 blk(32, R64_Y), grd((L0.nx + 31) / 32, (L0.nz + R64_Y * R64_ROWS - 1) / (R64_Y * R64_ROWS), nrhs);
+    FgDev fg = {};
+    if (fgp) fg = *fgp;
     if (L0.rho)
         k_resid64<TI, true><<<grd, blk, 0, s>>>(L0, npml, layer_coef(npml, amax), w2, f, u, rin, partials, pstride,
-                                                st, tol, inner_floor, inner_fac, first);
+                                                st, tol, inner_floor, inner_fac, first, fg);
     else
         k_resid64<TI, false><<<grd, blk, 0, s>>>(L0, npml, layer_coef(npml, amax), w2, f, u, rin, partials, pstride,
-                                                 st, tol, inner_floor, inner_fac, first);
+                                                 st, tol, inner_floor, inner_fac, first, fg);
 }
-template void launch_resid64<float>(const LevelDev&, int, double, const double*, const double*, const double*, float*, double*, int, RhsState*, double, double, double, int, int, cudaStream_t);
-template void launch_resid64<double>(const LevelDev&, int, double, const double*, const double*, const double*, double*, double*, int, RhsState*, double, double, double, int, int, cudaStream_t);
+template void launch_resid64<float>(const LevelDev&, int, double, const double*, const double*, const double*, float*, double*, int, RhsState*, double, double, double, int, int, cudaStream_t, const FgDev*);
+template void launch_resid64<double>(const LevelDev&, int, double, const double*, const double*, const double*, double*, double*, int, RhsState*, double, double, double, int, int, cudaStream_t, const FgDev*);
 
 // u += x for the right-hand sides still refining; an inner solve whose residual
 // overflowed (a divergent unpreconditioned iteration) leaves u, the best iterate

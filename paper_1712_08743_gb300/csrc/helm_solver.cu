@@ -467,8 +467,8 @@ template <typename T>
 static int alloc_inner(const SolveCtx& c, Inner<T>& w) {
     const helm_model* m = c.m;
     const size_t n = c.m->n(), vb = sizeof(T) * 2 * n * c.nrhs;
-    TRY_ALLOC(w.x, vb, c.s);
     if (c.o.krylov == HELM_KRYLOV_BICGSTAB) {      // FGMRES keeps its vectors in FgBufs
+        TRY_ALLOC(w.x, vb, c.s);
         TRY_ALLOC(w.r, vb, c.s); TRY_ALLOC(w.rh, vb, c.s);
         TRY_ALLOC(w.p, vb, c.s); TRY_ALLOC(w.v, vb, c.s); TRY_ALLOC(w.sv, vb, c.s);
         TRY_ALLOC(w.t, vb, c.s); TRY_ALLOC(w.ph, vb, c.s); TRY_ALLOC(w.shv, vb, c.s);
@@ -617,15 +617,14 @@ static int alloc_fg(const SolveCtx& c, FgBufs<T>& f) {
     return HELM_OK;
 }
 
-// One FGMRES cycle of at most m Arnoldi steps from a zero guess on rin; the
-// correction is left in w.x.
+// One FGMRES cycle of at most m Arnoldi steps from a zero guess on rin (its state set up by the
+// residual kernel); the correction is added to u64.
 template <typename T>
-static void fgmres_cycle(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* rin) {
+static void fgmres_cycle(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* rin, double* u64) {
     const size_t n = c.m->n(), vs = n * c.nrhs;
     const int m = f.dev.m, ro = c.o.reorth;
     T* V = f.V.template as<T>();
     T* Z = f.Z.template as<T>();
-    launch_fg_norm<T>(rin, c.partials, c.pstride, c.st, f.dev, c.nactive, n, c.nrhs, c.s);
     launch_fg_scale<T>(rin, V, c.st, f.dev, n, c.nrhs, c.s);
     bool pending = false;   // a column finish runs on the side stream
     for (int j = 0; j < m; ++j) {
@@ -666,20 +665,18 @@ static void fgmres_cycle(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* 
         pending = true;
     }
     if (pending) cudaStreamWaitEvent(c.s, c.ev_join, 0);
-    launch_fg_backsolve(c.st, f.dev, c.nrhs, c.s);
-    launch_fg_update<T>(Z, vs, w.x.template as<T>(), c.st, f.dev, n, c.nrhs, c.s);
+    launch_fg_update<T>(Z, vs, u64, c.st, f.dev, n, c.nrhs, c.s);
 }
 
 template <typename T>
-static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* rin, cudaGraphExec_t* graph,
-                        int* iters_done) {
+static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* rin, double* u64,
+                        cudaGraphExec_t* graph, int* iters_done) {
     NvtxRange nv("fgmres cycle");
-    HELM_CUDA_TRY(cudaMemsetAsync(c.nactive, 0, sizeof(int), c.s));
     if (c.o.use_graphs) {
         if (*graph == nullptr) {
             cudaGraph_t g;
             HELM_CUDA_TRY(cudaStreamBeginCapture(c.s, cudaStreamCaptureModeThreadLocal));
-            fgmres_cycle<T>(c, w, f, rin);
+            fgmres_cycle<T>(c, w, f, rin, u64);
             cudaError_t e = cudaStreamEndCapture(c.s, &g);
             if (e != cudaSuccess) { set_last_error(cudaGetErrorString(e)); return HELM_E_CUDA; }
             e = cudaGraphInstantiate(graph, g, 0);
@@ -688,10 +685,10 @@ static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* r
         }
         HELM_CUDA_TRY(cudaGraphLaunch(*graph, c.s));
     } else {
-        fgmres_cycle<T>(c, w, f, rin);
+        fgmres_cycle<T>(c, w, f, rin, u64);
     }
     const int m = f.dev.m;
-    count_launches(4 + (unsigned long long)m * ((c.o.precond == HELM_PRECOND_NONE ? 1 : mg_kernels_per_apply(c.m, sizeof(T) == 8, c.lf, c.ld, c.fca ? c.fca_level : 0, c.nrhs)) +
+    count_launches(2 + (unsigned long long)m * ((c.o.precond == HELM_PRECOND_NONE ? 1 : mg_kernels_per_apply(c.m, sizeof(T) == 8, c.lf, c.ld, c.fca ? c.fca_level : 0, c.nrhs)) +
                                                 (c.o.reorth == HELM_REORTH_NEVER ? 3 : c.o.reorth == HELM_REORTH_ALWAYS ? 5 : 4)));
     HELM_CUDA_TRY(cudaGetLastError());
     *iters_done += m;
@@ -897,7 +894,7 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
     for (int outer = 0;; ++outer) {
         NvtxRange nv_outer("refinement step");
         launch_resid64<T>(L0, m->npml, m->alpha_max, c.w2, f64, u64, rin.as<T>(), c.partials, c.pstride, c.st, o.tol,
-                          floor_tol, inner_fac, outer == 0, nrhs, s);
+                          floor_tol, inner_fac, outer == 0, nrhs, s, fgm ? &fb.dev : nullptr);
         count_launches(1);
         HELM_CUDA_TRY(cudaGetLastError());
         HELM_CUDA_TRY(cudaMemcpyAsync(hs.data(), c.st, sizeof(RhsState) * nrhs, cudaMemcpyDeviceToHost, s));
@@ -957,7 +954,7 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         for (int b = 0; b < nrhs; ++b) outer_count[b] += hs[b].outer_active;
         // BiCGSTAB keeps its recurrence across refinement steps (residual replacement)
         bool inner_stall = false;
-        rc = fgm ? fgmres_inner<T>(c, w, fb, rin.as<T>(), &graph, &iters_done)
+        rc = fgm ? fgmres_inner<T>(c, w, fb, rin.as<T>(), u64, &graph, &iters_done)
                  : inner_solve<T>(c, w, rin.as<T>(), &graph, &iters_done, outer > 0 && !restart_inner,
                                   guard && !switched ? kStallIters : 0, &inner_stall);
         restart_inner = false;
@@ -965,8 +962,10 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         if (rc != HELM_OK) break;
         rc = check_fcycle(c, fcerr);   // a persistent cycle that gave up a barrier ends the solve
         if (rc != HELM_OK) break;
-        launch_refine<T>(w.x.template as<T>(), u64, c.st, n, nrhs, s);
-        count_launches(1);
+        if (!fgm) {   // an FGMRES cycle ends with its own update of u
+            launch_refine<T>(w.x.template as<T>(), u64, c.st, n, nrhs, s);
+            count_launches(1);
+        }
     }
     if (graph) cudaGraphExecDestroy(graph);
     if (rc != HELM_OK) return rc;
