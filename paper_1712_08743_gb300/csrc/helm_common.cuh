@@ -24,6 +24,25 @@ template <typename T> __device__ __forceinline__ cx<T> operator*(cx<T> a, cx<T> 
     return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
 }
 template <typename T> __device__ __forceinline__ cx<T> operator*(T s, cx<T> a) { return {s * a.re, s * a.im}; }
+// Sums and real multiples of complex values for kernels that are bound by the issue of
+// instructions: in FP32 both parts go through one packed instruction (two rounded
+// operations each, the same results as the scalar pair). Complex products stay scalar:
+// packed, they need the parts of one factor swapped and cost as many instructions.
+template <typename T> __device__ __forceinline__ cx<T> padd(cx<T> a, cx<T> b) { return a + b; }
+template <> __device__ __forceinline__ cx<float> padd(cx<float> a, cx<float> b) {
+    const float2 r = __fadd2_rn(make_float2(a.re, a.im), make_float2(b.re, b.im));
+    return {r.x, r.y};
+}
+template <typename T> __device__ __forceinline__ cx<T> pfma(T s, cx<T> a, cx<T> c) {   // s a + c
+    return {s * a.re + c.re, s * a.im + c.im};
+}
+template <> __device__ __forceinline__ cx<float> pfma(float s, cx<float> a, cx<float> c) {
+    const float2 r = __ffma2_rn(make_float2(s, s), make_float2(a.re, a.im), make_float2(c.re, c.im));
+    return {r.x, r.y};
+}
+template <typename T> __device__ __forceinline__ cx<T> cfma(cx<T> a, cx<T> b, cx<T> c) {   // a b + c
+    return {(c.re + a.re * b.re) - a.im * b.im, (c.im + a.re * b.im) + a.im * b.re};
+}
 template <typename T> __device__ __forceinline__ cx<T> conjx(cx<T> a) { return {a.re, -a.im}; }
 // Reciprocal of |b|^2 in complex division: the FP32 smoother and preconditioner
 // use the hardware approximate divide (max 2 ulp), FP64 keeps the IEEE divide.

@@ -401,6 +401,9 @@ __global__ void __launch_bounds__(256) k_dense_mirror(TriShape sh, T* minv) {
 // one slot, group g = [grp[g], grp[g+1])); one warp per row of the inverse, the
 // row held in registers (NR complex values per lane per chunk) and reused for
 // every right-hand side of the group, whose vectors are staged in shared memory.
+// Warps per block: as many rows as give every SM a block, at most 8. In FP64 the multiplications bound
+// it (two per clock and SM): 690 rows, two right-hand sides, 41 us in 87 blocks of 8 rows with products
+// and sums apart, 23 us in 138 blocks of 5 with fused ones.
 template <typename T, int NR>
 __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict__ minv, const int* __restrict__ slot,
                                                       const int* __restrict__ grp, int maxg, const T* f, T* e,
@@ -409,7 +412,7 @@ __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict
     cx<T>* fs = reinterpret_cast<cx<T>*>(cd_smem);   // [group][n]
     pdl_trigger();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int row = blockIdx.x * 8 + warp;
+    const int row = blockIdx.x * (blockDim.x >> 5) + warp;
     const int g = blockIdx.y;
     const int b0 = grp[g], b1 = grp[g + 1];
     const T* Mr = minv + 2 * ((size_t)slot[b0] * n * n + (size_t)min(row, n - 1) * n);
@@ -446,8 +449,8 @@ __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict
                 const int j = c0 + lane + 32 * k;
                 if (j < n) {
                     const cx<T> v = fv[j];
-                    are[r] += rv[k].re * v.re - rv[k].im * v.im;
-                    aim[r] += rv[k].re * v.im + rv[k].im * v.re;
+                    are[r] = fma(-rv[k].im, v.im, fma(rv[k].re, v.re, are[r]));
+                    aim[r] = fma(rv[k].im, v.re, fma(rv[k].re, v.im, aim[r]));
                 }
             }
         }
@@ -533,7 +536,8 @@ void launch_coarse_dense(int n, const T* minv, const int* slot, const int* grp, 
         return true;
     }();
     (void)attr;
-    launch_pdl(k_coarse_dense<T, NR>, dim3((n + 7) / 8, ngroups), dim3(256), smem, s, n, minv, slot, grp, maxg, f, e,
+    const int warps = std::min(8, std::max(1, (int)(((size_t)n * ngroups + 151) / 152)));
+    launch_pdl(k_coarse_dense<T, NR>, dim3((n + warps - 1) / warps, ngroups), dim3(32 * warps), smem, s, n, minv, slot, grp, maxg, f, e,
                accumulate, st);
 }
 template void launch_coarse_dense<float>(int, const float*, const int*, const int*, int, int, const float*, float*,

@@ -199,10 +199,13 @@ __global__ void __launch_bounds__(AP_X * AP_Y) k_apply(LevelDev L, int npml, T a
             else if (ix + 1 >= nx) r = cx<T>(0, 0);
             const int d = max(max(dxd, max(npml - z, z - (nz - 1 - npml))), 0);
             const T s = hw * mm[k];
-            const T sa = s * (acoef * (T)(d * d));
             const T dd = T(4) - s;
-            cx<T> acc(dd * cur.re - sa * cur.im, dd * cur.im + sa * cur.re);
+            cx<T> acc(dd * cur.re, dd * cur.im);
             acc = acc - ((l + r) + (v[k] + v[k + 2]));
+            if (d > 0) {
+                const T sa = s * (acoef * (T)(d * d));
+                acc = cx<T>(acc.re - sa * cur.im, acc.im + sa * cur.re);
+            }
             stc(yb, i, scale * acc);
         }
     }
@@ -749,7 +752,9 @@ void launch_bicg_s(const T* r, const T* v, T* sv, const RhsState* st, size_t n, 
     launch_pdl(k_bicg_s<T>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, r, v, sv, st, n);
 }
 
-template <typename T>
+// x += alpha p^ + omega s^, r = s - omega t and the sums for the next scalars. SAME: s^ is s itself (no
+// preconditioner, or x holds the correction before the preconditioner), read once.
+template <typename T, bool SAME>
 __global__ void __launch_bounds__(256) k_bicg_xr(T* x, const T* __restrict__ ph, const T* __restrict__ shv,
                                                  const T* __restrict__ sv, const T* __restrict__ t,
                                                  const T* __restrict__ rh, T* r, double* partials, int pstride,
@@ -770,8 +775,9 @@ __global__ void __launch_bounds__(256) k_bicg_xr(T* x, const T* __restrict__ ph,
     T a0 = 0, a1 = 0, a2 = 0;   // <rh, r> (re, im), <r, r>
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         cx<T> xv = ldcc(x, off + i);
-        stc(x, off + i, xv + al * ldc(ph, off + i) + om * ldc(shv, off + i));
-        cx<T> rn = ldc(sv, off + i) - om * ldc(t, off + i);
+        const cx<T> s = ldc(sv, off + i);
+        stc(x, off + i, xv + al * ldc(ph, off + i) + om * (SAME ? s : ldc(shv, off + i)));
+        cx<T> rn = s - om * ldc(t, off + i);
         stc(r, off + i, rn);
         cx<T> q = ldc(rh, off + i);
         a0 += q.re * rn.re + q.im * rn.im;
@@ -815,9 +821,10 @@ __global__ void __launch_bounds__(256) k_bicg_xr(T* x, const T* __restrict__ ph,
 template <typename T>
 void launch_bicg_xr(T* x, const T* ph, const T* shv, const T* sv, const T* t, const T* rh, T* r, double* partials,
                     int pstride, RhsState* st, int* nactive, size_t n, int nrhs, cudaStream_t s) {
-    ProfScope prof(PK_BICG_XR, (int)n, 1, (double)n * nrhs * 16.0 * sizeof(T), s);
-    launch_pdl(k_bicg_xr<T>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, x, ph, shv, sv, t, rh, r, partials, pstride, st,
-               nactive, n);
+    const bool same = shv == sv;
+    ProfScope prof(PK_BICG_XR, (int)n, 1, (double)n * nrhs * (same ? 14.0 : 16.0) * sizeof(T), s);
+    launch_pdl(same ? k_bicg_xr<T, true> : k_bicg_xr<T, false>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, x, ph, shv,
+               sv, t, rh, r, partials, pstride, st, nactive, n);
 }
 
 // ===================================================== Galerkin operators
@@ -1225,7 +1232,8 @@ template <typename T> __device__ __forceinline__ cx<T> sh_dn(cx<T> a) {
 // columns. The warp walks down the fine rows of `ks` coarse rows two at a time,
 // holding u1 of three rows in registers and loading two rows ahead; the
 // neighbour columns across a lane boundary come by shuffle. r is zero outside
-// the grid.
+// the grid. 320 right-hand sides of 441 x 241 in FP32: packed sums 57.3 -> 54.9 us, two steps per loop
+// (the rotating rows need no moves) -> 52 us.
 constexpr int RM_COLS = 30;   // coarse columns per warp
 
 // The marching loop; EDGE = false when every row and column the warp touches
@@ -1258,8 +1266,8 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
     auto resid = [&](int z, const Row& rz, cx<T> a0, cx<T> a1, cx<T> c0v, cx<T> c1v, cx<T> d0v, cx<T> d1v,
                      cx<T>& r0, cx<T>& r1) {
         const cx<T> wl = sh_up(c1v), er = sh_dn(c0v);
-        r0 = omw * rz.f0 + (a0 + d0v) + (wl + c1v);
-        r1 = omw * rz.f1 + (a1 + d1v) + (c0v + er);
+        r0 = pfma(omw, rz.f0, padd(padd(a0, d0v), padd(wl, c1v)));
+        r1 = pfma(omw, rz.f1, padd(padd(a1, d1v), padd(c0v, er)));
         if (EDGE) {
             const bool zin = z < nz;
             if (!(zin && in0)) r0 = cx<T>(0, 0);
@@ -1267,13 +1275,14 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
         }
     };
     // horizontal full weighting at the centre column: r(2I) + 2 r(2I+1) + r(2I+2)
-    auto hsum = [&](cx<T> r0, cx<T> r1) -> cx<T> { return (r0 + sh_dn(r0)) + T(2) * r1; };
+    auto hsum = [&](cx<T> r0, cx<T> r1) -> cx<T> { return pfma(T(2), r1, padd(r0, sh_dn(r0))); };
     const bool wr = lane >= 1 && lane <= RM_COLS && I < cnx;
 
     Row A = ld(2 * K0 - 1), B = ld(2 * K0), C = ld(2 * K0 + 1), D = ld(2 * K0 + 2);
     cx<T> ua0 = u1of(A.f0, A.m0), ua1 = u1of(A.f1, A.m1);   // u1 of row 2K-1
     cx<T> ub0 = u1of(B.f0, B.m0), ub1 = u1of(B.f1, B.m1);   // u1 of row 2K
     cx<T> acc(0, 0);
+#pragma unroll 2   // a row pair's registers become the next pair's without moves
     for (int K = K0; K < K1; ++K) {
         // held: u1 of rows 2K-1, 2K, f of row 2K (B); raw rows 2K+1 (C), 2K+2 (D)
         const Row E = ld(2 * K + 3), F = ld(2 * K + 4);
@@ -1284,10 +1293,10 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
         resid(2 * K + 1, C, ub0, ub1, uc0, uc1, ud0, ud1, s0, s1);
         const cx<T> h0 = hsum(r0, r1), h1 = hsum(s0, s1);
         if (K > K0) {
-            acc = acc + h0;   // completes coarse row K - 1
+            acc = padd(acc, h0);   // completes coarse row K - 1
             if (wr) stc(fcb, (size_t)(K - 1) * cnx + I, T(0.25) * acc);
         }
-        acc = h0 + T(2) * h1;
+        acc = pfma(T(2), h1, h0);
         ua0 = uc0; ua1 = uc1; ub0 = ud0; ub1 = ud1;
         B = D; C = E; D = F;
     }
@@ -1326,10 +1335,12 @@ __global__ void __launch_bounds__(256) k_restrict(LevelDev Lf, LevelDev Lc, cons
 
 // Rows per block of the marching kernels: long segments amortise the rows
 // recomputed at segment ends; short ones give enough warps when the batch is
-// small (aim: 32 warps per SM on 152 SMs).
-inline int march_rows(int col_warps, int rows, int nrhs, int longest) {
+// small (aim: 32 warps per SM on 152 SMs). FP64 issues an instruction in 16 cycles of an SM: 8 warps
+// keep its pipe busy, and more of them only add rows that are computed twice.
+template <typename T> constexpr unsigned kMarchWarps = sizeof(T) == 4 ? 32 : 8;
+inline int march_rows(int col_warps, int rows, int nrhs, int longest, unsigned warps) {
     int zs = longest;
-    while (zs > 4 && (size_t)col_warps * ((rows + zs - 1) / zs) * nrhs < 152u * 32u) zs /= 2;
+    while (zs > 4 && (size_t)col_warps * ((rows + zs - 1) / zs) * nrhs < 152u * warps) zs /= 2;
     return zs;
 }
 
@@ -1345,7 +1356,7 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
                    s);
     if (Lf.m2 && !Lf.rho) {   // finest constant-density level; a density level is stored like a coarse one
         const int cw = (Lc.nx + RM_COLS - 1) / RM_COLS;
-        const int ks = march_rows(cw, Lc.nz, nrhs, 16);
+        const int ks = march_rows(cw, Lc.nz, nrhs, 16, kMarchWarps<T>);
         dim3 grd((cw + 7) / 8, (Lc.nz + ks - 1) / ks, nrhs);
         launch_pdl(k_restrict<T>, grd, dim3(256), 0, s, Lf, Lc, w2, (T)b1, (T)b2, (T)wj, f, fc, st, ks);
     } else {
@@ -1367,6 +1378,12 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
 // two at a time (u2 of rows 2K, 2K+1; u3 of rows 2K-1, 2K; outputs of rows
 // 2K-2, 2K-1), holding the rows it still needs in registers and loading two
 // rows ahead; neighbours across a lane boundary come by shuffle.
+// FP32 on 320 right-hand sides of 441 x 241: 16 warps per SM (registers) that issue in 50 to 70 % of
+// the cycles, waiting for loads otherwise. The damping terms only where a row or the warp's columns have
+// any, and packed sums: 142 -> 128 us. A cap of 128 registers for mode 1 spills (137 us). FP64 is bound
+// by its arithmetic at two results per clock and SM: the first step's unused u3, the rows above
+// the segment and the second divide of odd rows left out, and longer segments (march_rows): 80 -> 61 us on 241 x
+// 191 with two right-hand sides. In FP32 the skipped rows cost more in scheduling than they save (156 us).
 constexpr int PM_COLS = 60;   // fine output columns per warp
 
 template <typename T, int MODE, bool EDGE>
@@ -1374,7 +1391,7 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
                                               int npml, T acoef, T hw, T b1, T b2, T wj, const T* __restrict__ fb,
                                               const T* __restrict__ eb, const T* __restrict__ ab,
                                               const T* __restrict__ m2, T* __restrict__ ob, T* __restrict__ yb,
-                                              int accumulate, T& d0, T& d1, T& d2) {
+                                              int accumulate, bool wout, T& d0, T& d1, T& d2) {
     const int c0 = 2 * J;
     const bool in0 = !EDGE || (c0 >= 0 && c0 < nx), in1 = !EDGE || (c0 + 1 >= 0 && c0 + 1 < nx);
     const bool ein = !EDGE || (J >= 0 && J < cnx);
@@ -1410,13 +1427,14 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
     // u2 of row z at both columns; ev = e(K, J) of the coarse rows above and
     // below (equal for odd z): column 2J + 1 takes e(J), column 2J the mean of
     // e(J - 1) (lower lane) and e(J)
-    auto u2row = [&](int z, const Row& r, const ERow& ea, const ERow& ec2, cx<T>& p0, cx<T>& p1) {
-        const cx<T> ev = T(0.5) * (ea.e + ec2.e);
+    auto u2row = [&](int z, const Row& r, const ERow& ea, const ERow& ec2, cx<T> i0, cx<T> i1, cx<T>& p0,
+                     cx<T>& p1) {
+        const cx<T> ev = T(0.5) * padd(ea.e, ec2.e);
         const cx<T> up = sh_up(ev);
-        const cx<T> left = lane == 0 ? T(0.5) * (ea.w + ec2.w) : up;
-        const cx<T> pe0 = T(0.5) * (left + ev);
-        p0 = dinv(r.m0) * r.f0 + pe0;
-        p1 = dinv(r.m1) * r.f1 + ev;
+        const cx<T> left = lane == 0 ? T(0.5) * padd(ea.w, ec2.w) : up;
+        const cx<T> pe0 = T(0.5) * padd(left, ev);
+        p0 = cfma(i0, r.f0, pe0);
+        p1 = cfma(i1, r.f1, ev);
         if (EDGE) {
             const bool zin = z >= 0 && z < nz;
             if (!(zin && in0)) p0 = cx<T>(0, 0);
@@ -1424,11 +1442,11 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
         }
     };
     // u3 of row z from u2 of rows z-1 (a), z (c), z+1 (d)
-    auto u3row = [&](int z, const Row& r, cx<T> a0, cx<T> a1, cx<T> c0v, cx<T> c1v, cx<T> d0v, cx<T> d1v,
+    auto u3row = [&](int z, const Row& r, cx<T> i0, cx<T> i1, cx<T> a0, cx<T> a1, cx<T> c0v, cx<T> c1v, cx<T> d0v, cx<T> d1v,
                      cx<T>& q0, cx<T>& q1) {
         const cx<T> wl = sh_up(c1v), er = sh_dn(c0v);
-        q0 = omw * c0v + dinv(r.m0) * (r.f0 + ((wl + c1v) + (a0 + d0v)));
-        q1 = omw * c1v + dinv(r.m1) * (r.f1 + ((c0v + er) + (a1 + d1v)));
+        q0 = pfma(omw, c0v, i0 * padd(r.f0, padd(padd(wl, c1v), padd(a0, d0v))));
+        q1 = pfma(omw, c1v, i1 * padd(r.f1, padd(padd(c0v, er), padd(a1, d1v))));
         if (EDGE) {
             const bool zin = z >= 0 && z < nz;
             if (!(zin && in0)) q0 = cx<T>(0, 0);
@@ -1437,16 +1455,21 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
     };
     // y = A u3 at row z (fine operator with damping) from u3 of rows z-1, z, z+1
     const int dx0 = max(npml - c0, c0 - (nx - 1 - npml)), dx1 = max(npml - c0 - 1, c0 + 1 - (nx - 1 - npml));
+    const bool damp = MODE != 0 && __any_sync(0xffffffffu, max(dx0, dx1) > 0);
     auto arow = [&](int z, const Row& r, cx<T> a0, cx<T> a1, cx<T> c0v, cx<T> c1v, cx<T> d0v, cx<T> d1v,
                     cx<T>& y0, cx<T>& y1) {
         const cx<T> wl = sh_up(c1v), er = sh_dn(c0v);
         const int dz = max(npml - z, z - (nz - 1 - npml));
-        const int e0 = max(max(dx0, dz), 0), e1 = max(max(dx1, dz), 0);
         const T s0 = hw * r.m0, s1 = hw * r.m1;
-        const T a0s = s0 * (acoef * (T)(e0 * e0)), a1s = s1 * (acoef * (T)(e1 * e1));
-        const T g0 = T(4) - s0, g1 = T(4) - s1;
-        y0 = cx<T>(g0 * c0v.re - a0s * c0v.im, g0 * c0v.im + a0s * c0v.re) - ((wl + c1v) + (a0 + d0v));
-        y1 = cx<T>(g1 * c1v.re - a1s * c1v.im, g1 * c1v.im + a1s * c1v.re) - ((c0v + er) + (a1 + d1v));
+        const cx<T> n0 = padd(padd(wl, c1v), padd(a0, d0v)), n1 = padd(padd(c0v, er), padd(a1, d1v));
+        y0 = pfma(T(4) - s0, c0v, T(-1) * n0);
+        y1 = pfma(T(4) - s1, c1v, T(-1) * n1);
+        if (damp || dz > 0) {   // uniform in the warp
+            const int e0 = max(max(dx0, dz), 0), e1 = max(max(dx1, dz), 0);
+            const T a0s = s0 * (acoef * (T)(e0 * e0)), a1s = s1 * (acoef * (T)(e1 * e1));
+            y0 = cx<T>(y0.re - a0s * c0v.im, y0.im + a0s * c0v.re);
+            y1 = cx<T>(y1.re - a1s * c1v.im, y1.im + a1s * c1v.re);
+        }
     };
     auto lda = [&](int z, cx<T>& q0, cx<T>& q1) {
         const bool ok = outl && z >= Z0 && z < Z1;
@@ -1464,6 +1487,10 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
     RA.f0 = RA.f1 = RB.f0 = RB.f1 = cx<T>(0, 0);
     RA.m0 = RA.m1 = RB.m0 = RB.m1 = T(0);
     Row RC = ld(2 * Ks), RD = ld(2 * Ks + 1);
+    // FP64 keeps wj D^-1 of the odd row for the next step (its divide is a dozen of the instructions that
+    // bound the kernel); FP32 forms it again, which is cheaper than the registers
+    constexpr bool KEEP = sizeof(T) == 8 && MODE != 1;
+    cx<T> ib0(0, 0), ib1(0, 0);
     ERow elo = erow(Ks - 1), ehi = erow(Ks);
     cx<T> qr0(0, 0), qr1(0, 0), qs0(0, 0), qs1(0, 0);   // mode 1: shadow residual of the output rows
     if constexpr (MODE == 1) { lda(2 * Ks - 2, qr0, qr1); lda(2 * Ks - 1, qs0, qs1); }
@@ -1473,13 +1500,19 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
         cx<T> qn0(0, 0), qn1(0, 0), qm0(0, 0), qm1(0, 0);
         if constexpr (MODE == 1) { lda(2 * K, qn0, qn1); lda(2 * K + 1, qm0, qm1); }
         cx<T> pc0, pc1, pd0, pd1, qc0, qc1, qd0, qd1;
-        u2row(2 * K, RC, elo, ehi, pc0, pc1);       // even row: mean of e(K-1), e(K)
-        u2row(2 * K + 1, RD, ehi, ehi, pd0, pd1);   // odd row: e(K)
-        u3row(2 * K - 1, RB, pa0, pa1, pb0, pb1, pc0, pc1, qc0, qc1);
-        u3row(2 * K, RC, pb0, pb1, pc0, pc1, pd0, pd1, qd0, qd1);
+        const cx<T> ic0 = dinv(RC.m0), ic1 = dinv(RC.m1), id0 = dinv(RD.m0), id1 = dinv(RD.m1);
+        u2row(2 * K, RC, elo, ehi, ic0, ic1, pc0, pc1);       // even row: mean of e(K-1), e(K)
+        u2row(2 * K + 1, RD, ehi, ehi, id0, id1, pd0, pd1);   // odd row: e(K)
+        qc0 = qc1 = qd0 = qd1 = cx<T>(0, 0);
+        if (sizeof(T) == 4 || K > Ks) {   // the first step prepares u2 only
+            if constexpr (!KEEP) { ib0 = dinv(RB.m0); ib1 = dinv(RB.m1); }
+            u3row(2 * K - 1, RB, ib0, ib1, pa0, pa1, pb0, pb1, pc0, pc1, qc0, qc1);
+            u3row(2 * K, RC, ic0, ic1, pb0, pb1, pc0, pc1, pd0, pd1, qd0, qd1);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int z = 2 * K - 2 + h;
+            if (sizeof(T) == 8 && z < Z0) break;   // rows of the segment above
             const cx<T> c0v = h ? qc0 : qb0, c1v = h ? qc1 : qb1;
             const bool wr = outl && z >= Z0 && z < Z1;
             const int i = z * nx + c0;
@@ -1493,8 +1526,12 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
                 if (h) arow(z, RB, qb0, qb1, qc0, qc1, qd0, qd1, y0, y1);
                 else arow(z, RA, qa0, qa1, qb0, qb1, qc0, qc1, y0, y1);
                 if (wr) {
-                    if (in0) { stc(ob, i, c0v); stc(yb, i, y0); }
-                    if (in1) { stc(ob, i + 1, c1v); stc(yb, i + 1, y1); }
+                    if (MODE == 3 || wout) {
+                        if (in0) stc(ob, i, c0v);
+                        if (in1) stc(ob, i + 1, c1v);
+                    }
+                    if (in0) stc(yb, i, y0);
+                    if (in1) stc(yb, i + 1, y1);
                     if (!in0) y0 = cx<T>(0, 0);
                     if (!in1) y1 = cx<T>(0, 0);
                     if constexpr (MODE == 1) {          // <rh, v>
@@ -1513,6 +1550,7 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
         pa0 = pc0; pa1 = pc1; pb0 = pd0; pb1 = pd1;
         qa0 = qc0; qa1 = qc1; qb0 = qd0; qb1 = qd1;
         RA = RC; RB = RD; RC = RE; RD = RF;
+        if constexpr (KEEP) { ib0 = id0; ib1 = id1; }
         elo = ehi; ehi = enx;
         qr0 = qn0; qr1 = qn1; qs0 = qm0; qs1 = qm1;
     }
@@ -1551,10 +1589,10 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
                           Z0 / 2 - 2 < 0 || Z1 / 2 + 2 >= cnz;
         if (edge)
             prolong_march<T, MODE, true>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
-                                         eb, ab, m2, ob, yb, accumulate, d0, d1, d2);
+                                         eb, ab, m2, ob, yb, accumulate, out != nullptr, d0, d1, d2);
         else
             prolong_march<T, MODE, false>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
-                                          eb, ab, m2, ob, yb, accumulate, d0, d1, d2);
+                                          eb, ab, m2, ob, yb, accumulate, out != nullptr, d0, d1, d2);
     }
     if constexpr (MODE == 0 || MODE == 3) return;
     else {
@@ -1585,9 +1623,9 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
 }
 
 // Grid of the marching prolongation for a fine level of nx x nz nodes.
-inline dim3 prolong_grid(int nx, int nz, int nrhs, int longest, int* zs) {
+inline dim3 prolong_grid(int nx, int nz, int nrhs, int longest, unsigned warps, int* zs) {
     const int cw = (nx + PM_COLS - 1) / PM_COLS;
-    *zs = march_rows(cw, nz, nrhs, longest);
+    *zs = march_rows(cw, nz, nrhs, longest, warps);
     return dim3((cw + PM_WARPS - 1) / PM_WARPS, (nz + *zs - 1) / *zs, nrhs);
 }
 
@@ -1613,7 +1651,7 @@ void launch_prolong(int mode, const LevelDev& Lf, const LevelDev& Lc, int npml, 
     }
     // finest level: the tile choice is the longest row segment (16 or 32 rows)
     int zs = 0;
-    const dim3 grd = prolong_grid(Lf.nx, Lf.nz, nrhs, tile == 0 ? 16 : 32, &zs);
+    const dim3 grd = prolong_grid(Lf.nx, Lf.nz, nrhs, tile == 0 ? 16 : 32, kMarchWarps<T>, &zs);
     if (mode == 0)
         launch_pdl(k_prolong<T, 0>, grd, dim3(32 * PM_WARPS), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);

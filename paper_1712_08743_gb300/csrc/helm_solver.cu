@@ -113,7 +113,16 @@ struct SolveCtx {
     int fca_level = 0, fca_grid = 0;
     cudaStream_t side = nullptr;    // FGMRES: the Hessenberg column finish runs here
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    bool late_precond = false;      // BiCGSTAB sums its correction before the preconditioner
 };
+
+// BiCGSTAB's correction x = sum of alpha p^ + omega s^ with p^ = V(p), s^ = V(s): V is linear and the
+// same for a whole inner solve, so the sum can be taken over p and s and V applied to it once,
+// when the inner solve ends. The iterations then neither write p^ and s^ nor read p^, 3 of their 24
+// passes over a vector. The extra cycle costs as much as half an iteration, which is more than that
+// where vectors stay in L2 or launches bound the solve (six refinements of a 101 x 101 solve:
+// 0.3 of 4.7 ms); so it is done once the nine vectors of the solve exceed the 129 MB of L2.
+constexpr size_t kLatePrecondBytes = (size_t)16 << 20;   // bytes of one vector of the batch
 
 // The second stream and events of an FGMRES solve.
 struct SideStream {
@@ -471,7 +480,10 @@ static int alloc_inner(const SolveCtx& c, Inner<T>& w) {
         TRY_ALLOC(w.x, vb, c.s);
         TRY_ALLOC(w.r, vb, c.s); TRY_ALLOC(w.rh, vb, c.s);
         TRY_ALLOC(w.p, vb, c.s); TRY_ALLOC(w.v, vb, c.s); TRY_ALLOC(w.sv, vb, c.s);
-        TRY_ALLOC(w.t, vb, c.s); TRY_ALLOC(w.ph, vb, c.s); TRY_ALLOC(w.shv, vb, c.s);
+        TRY_ALLOC(w.t, vb, c.s);
+        if (!c.late_precond || m->vd) {   // a density model applies A to p^ and s^ in a kernel of its own
+            TRY_ALLOC(w.ph, vb, c.s); TRY_ALLOC(w.shv, vb, c.s);
+        }
     }
     return alloc_levels<T>(c.m, c.s, c.nrhs, w, c.ld > 0 ? c.ld : c.m->tail_level(sizeof(T) == 8));
 }
@@ -504,13 +516,16 @@ static void bicg_iteration(const SolveCtx& c, Inner<T>& w) {
     vcycle<T>(c, w, p, ph, 1, v, rh);              // p^ = V(p), v = A p^, alpha
     launch_bicg_s<T>(r, v, sv, c.st, n, c.nrhs, c.s);
     vcycle<T>(c, w, sv, shv, 2, t, nullptr);       // s^ = V(s), t = A s^, omega
-    launch_bicg_xr<T>(x, ph, shv, sv, t, rh, r, c.partials, c.pstride, c.st, c.nactive, n, c.nrhs, c.s);
+    launch_bicg_xr<T>(x, c.late_precond ? p : ph, c.late_precond ? sv : shv, sv, t, rh, r, c.partials, c.pstride,
+                      c.st, c.nactive, n, c.nrhs, c.s);
 }
 
 // Inner BiCGSTAB on rin for the right-hand sides whose outer step is active.
-// Leaves the correction in w.x. `graph` caches the captured iteration chunk.
+// *corr: where the correction is left (w.x, or w.t when V is applied to w.x last). `graph`
+// caches the captured iteration chunk.
 template <typename T>
-static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, cudaGraphExec_t* graph, int* iters_done,
+static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, const T** corr, cudaGraphExec_t* graph,
+                       int* iters_done,
                        bool resume, int guard_iters, bool* stalled) {
     const size_t n = c.m->n();
     HELM_CUDA_TRY(cudaMemsetAsync(c.nactive, 0, sizeof(int), c.s));
@@ -576,6 +591,15 @@ static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, cudaGraphEx
             }
             if (stall) { *stalled = true; break; }
         }
+    }
+    *corr = w.x.template as<T>();
+    if (c.late_precond) {
+        SolveCtx all = c;
+        all.st = nullptr;   // every right-hand side: those that have converged are no longer active
+        vcycle<T>(all, w, w.x.template as<T>(), w.t.template as<T>(), 0, nullptr, nullptr);
+        count_launches(mg_kernels_per_apply(c.m, sizeof(T) == 8, c.lf, c.ld, c.fca ? c.fca_level : 0, c.nrhs) -
+                       (c.m->vd ? 1 : 0));
+        *corr = w.t.template as<T>();
     }
     HELM_CUDA_TRY(cudaGetLastError());
     *iters_done += done;
@@ -843,6 +867,8 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         c.maxg = q.maxg;
     };
     use_coarse(*cs);
+    c.late_precond = o.krylov == HELM_KRYLOV_BICGSTAB && o.precond != HELM_PRECOND_NONE &&
+                     sizeof(T) * 2 * n * nrhs >= kLatePrecondBytes;
     Inner<T> w;
     rc = alloc_inner<T>(c, w);
     if (rc != HELM_OK) return rc;
@@ -954,8 +980,9 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         for (int b = 0; b < nrhs; ++b) outer_count[b] += hs[b].outer_active;
         // BiCGSTAB keeps its recurrence across refinement steps (residual replacement)
         bool inner_stall = false;
+        const T* corr = nullptr;
         rc = fgm ? fgmres_inner<T>(c, w, fb, rin.as<T>(), u64, &graph, &iters_done)
-                 : inner_solve<T>(c, w, rin.as<T>(), &graph, &iters_done, outer > 0 && !restart_inner,
+                 : inner_solve<T>(c, w, rin.as<T>(), &corr, &graph, &iters_done, outer > 0 && !restart_inner,
                                   guard && !switched ? kStallIters : 0, &inner_stall);
         restart_inner = false;
         if (inner_stall) force_switch = true;
@@ -963,7 +990,7 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
         rc = check_fcycle(c, fcerr);   // a persistent cycle that gave up a barrier ends the solve
         if (rc != HELM_OK) break;
         if (!fgm) {   // an FGMRES cycle ends with its own update of u
-            launch_refine<T>(w.x.template as<T>(), u64, c.st, n, nrhs, s);
+            launch_refine<T>(corr, u64, c.st, n, nrhs, s);
             count_launches(1);
         }
     }
