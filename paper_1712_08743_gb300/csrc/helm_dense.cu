@@ -399,26 +399,27 @@ __global__ void __launch_bounds__(256) k_dense_mirror(TriShape sh, T* minv) {
 
 // e_b (+)= M_d^-1 f_b for the right-hand sides of one group (consecutive RHS of
 // one slot, group g = [grp[g], grp[g+1])); one warp per row of the inverse, the
-// row held in registers (NR complex values per lane per chunk) and reused for
+// row held in registers (NR complex values per lane) and reused for
 // every right-hand side of the group, whose vectors are staged in shared memory.
 // Warps per block: as many rows as give every SM a block, at most 8. In FP64 the multiplications bound
-// it (two per clock and SM): 690 rows, two right-hand sides, 41 us in 87 blocks of 8 rows with products
-// and sums apart, 23 us in 138 blocks of 5 with fused ones.
+// it (a quarter of an SM does one lane in two clocks): 690 rows, two right-hand sides, 41 us in 87 blocks of
+// 8 rows with products and sums apart, 23 us in 138 blocks of 5 with fused ones, 16 us with the whole row and
+// four values of f in flight per thread; complex64, 966 rows, four right-hand sides, 13.4 -> 12.1 us.
 template <typename T, int NR>
 __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict__ minv, const int* __restrict__ slot,
                                                       const int* __restrict__ grp, int maxg, const T* f, T* e,
                                                       int accumulate, const RhsState* st) {
     extern __shared__ __align__(16) unsigned char cd_smem[];
     cx<T>* fs = reinterpret_cast<cx<T>*>(cd_smem);   // [group][n]
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int row = blockIdx.x * (blockDim.x >> 5) + warp;
     const int g = blockIdx.y;
     const int b0 = grp[g], b1 = grp[g + 1];
     const T* Mr = minv + 2 * ((size_t)slot[b0] * n * n + (size_t)min(row, n - 1) * n);
-    constexpr int CH = 32 * NR;
+    static_assert(32 * NR >= kDenseMaxPoints, "a row of the inverse in one warp's registers");
     cx<T> rv[NR];
-    // the first chunk of this warp's row is model data: load it before waiting on the previous kernel
+    // this warp's row is model data: load it before waiting on the previous kernel
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
         const int j = lane + 32 * k;
@@ -426,32 +427,35 @@ __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict
     }
     pdl_wait();
     const int nb = b1 - b0;
-    for (int idx = threadIdx.x; idx < nb * n; idx += blockDim.x) fs[idx] = ldcc(f, (size_t)b0 * n + idx);
+    for (int idx = threadIdx.x; idx < nb * n; idx += 4 * blockDim.x) {   // four loads in flight
+        cx<T> q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = idx + k * blockDim.x;
+            q[k] = i < nb * n ? ldcc(f, (size_t)b0 * n + i) : cx<T>(0, 0);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = idx + k * blockDim.x;
+            if (i < nb * n) fs[i] = q[k];
+        }
+    }
     __syncthreads();
     if (row >= n) return;
     T are[8], aim[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) { are[r] = T(0); aim[r] = T(0); }
-    for (int c0 = 0; c0 < n; c0 += CH) {
-        if (c0 > 0) {
 #pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const int j = c0 + lane + 32 * k;
-                rv[k] = j < n ? ldc(Mr, j) : cx<T>(0, 0);
-            }
-        }
+    for (int r = 0; r < 8; ++r) {
+        if (r >= nb) break;
+        const cx<T>* fv = fs + (size_t)r * n;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if (r >= nb) break;
-            const cx<T>* fv = fs + (size_t)r * n;
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const int j = c0 + lane + 32 * k;
-                if (j < n) {
-                    const cx<T> v = fv[j];
-                    are[r] = fma(-rv[k].im, v.im, fma(rv[k].re, v.re, are[r]));
-                    aim[r] = fma(rv[k].im, v.re, fma(rv[k].re, v.im, aim[r]));
-                }
+        for (int k = 0; k < NR; ++k) {
+            const int j = lane + 32 * k;
+            if (j < n) {
+                const cx<T> v = fv[j];
+                are[r] = fma(-rv[k].im, v.im, fma(rv[k].re, v.re, are[r]));
+                aim[r] = fma(rv[k].im, v.re, fma(rv[k].re, v.im, aim[r]));
             }
         }
     }
@@ -526,7 +530,7 @@ template cudaError_t launch_dense_invert<double>(const LevelDev&, const double*,
 template <typename T>
 void launch_coarse_dense(int n, const T* minv, const int* slot, const int* grp, int ngroups, int maxg, const T* f,
                          T* e, int accumulate, const RhsState* st, cudaStream_t s) {
-    constexpr int NR = sizeof(T) == 4 ? 38 : 19;
+    constexpr int NR = (kDenseMaxPoints + 31) / 32;   // a row fits the registers, so that all of it is loaded ahead
     // the inverse of each group's slot once per group, f read and e written (and read when accumulating)
     ProfScope prof(PK_COARSE_DENSE, n, 1,
                    ((double)n * n * ngroups + (double)n * (2 + accumulate) * ngroups * maxg) * 2.0 * sizeof(T), s);

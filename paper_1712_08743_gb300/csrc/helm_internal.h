@@ -34,6 +34,7 @@ constexpr int kGalerkinCoefs = 10;   // per coarse node: G (c, e, n, ne, nw) the
 // the first level with at most this many nodes is solved exactly by its dense inverse
 // (few right-hand sides; see helm_dense.cu)
 constexpr int kDenseMaxPoints = 1200;
+constexpr int kVecBlocks = 4 * 152;   // blocks that the vector kernels of a small BiCGSTAB batch spread over
 constexpr int kDenseAutoMaxRhs = 16;   // HELM_COARSE_AUTO takes the dense level for batches up to this size
 // the cycle fuses consecutive Galerkin prolongations (launch_prolong2) for batches up to this size
 constexpr int kProlong2MaxRhs = kDenseAutoMaxRhs;
@@ -144,7 +145,12 @@ struct DBuf {
 };
 
 // Launch with programmatic stream serialization (the kernel must call pdl_wait
-// before reading anything an earlier kernel of the stream writes).
+// before reading anything an earlier kernel of the stream writes), which hides a launch
+// and the first loads of a kernel that takes a few microseconds. A grid of more than two full GPUs of
+// threads starts when the kernel before has ended: early, its blocks only take room and L2 from that
+// one (320 right-hand sides of 441 x 241: 273 -> 262 ms, 128: 234 -> 223 ms; a line at one GPU: 265 ms, as
+// it takes the 320 blocks of the tail too; none for any grid: one right-hand side of 1041 x 1041 209 -> 221 ms).
+constexpr size_t kPdlMaxThreads = (size_t)152 * 4096;
 template <typename... KArgs, typename... Args>
 void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -156,7 +162,7 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (size_t)grid.x * grid.y * grid.z * block.x * block.y * block.z <= kPdlMaxThreads ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

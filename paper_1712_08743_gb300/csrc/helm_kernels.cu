@@ -29,6 +29,12 @@ inline int grid1d(size_t n) {
     if (g > 2048) g = 2048;
     return (int)g;
 }
+// The same for the vector kernels of BiCGSTAB: a small batch has blocks of one node per thread
+// until there are four blocks per SM (p of two FP64 right-hand sides of 241 x 191: 10.0 -> 8.3 us).
+inline int grid_vec(size_t n, int nrhs) {
+    const size_t most = std::min<size_t>((n + 255) / 256, (kVecBlocks + nrhs - 1) / nrhs);
+    return (int)std::max<size_t>(grid1d(n), most);
+}
 
 }  // namespace
 
@@ -273,7 +279,7 @@ __global__ void __launch_bounds__(256) k_apply_dots(LevelDev L, int npml, T acoe
                                                     const T* __restrict__ aux, double* partials, int pstride,
                                                     RhsState* st, T scale) {
     __shared__ double shred[96];
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!rhs_active(st, b)) return;
@@ -620,7 +626,7 @@ template <typename T>
 void launch_bicg_init(const T* b, T* x, T* r, T* rh, T* p, T* v, double* partials, int pstride, RhsState* st,
                       int* nactive, size_t n, int nrhs, cudaStream_t s) {
     ProfScope prof(PK_BICG_INIT, (int)n, 1, (double)n * nrhs * 12.0 * sizeof(T), s);
-    k_bicg_init<T><<<dim3(grid1d(n), 1, nrhs), 256, 0, s>>>(b, x, r, rh, p, v, partials, pstride, st, nactive, n);
+    k_bicg_init<T><<<dim3(grid_vec(n, nrhs), 1, nrhs), 256, 0, s>>>(b, x, r, rh, p, v, partials, pstride, st, nactive, n);
 }
 
 // Residual replacement ("reliable update") between refinement steps: r is
@@ -696,7 +702,7 @@ template <typename T>
 void launch_bicg_resume(const T* rin, T* x, T* r, T* rh, T* p, T* v, double* partials, int pstride, RhsState* st,
                         int* nactive, size_t n, int nrhs, cudaStream_t s) {
     ProfScope prof(PK_BICG_RESUME, (int)n, 1, (double)n * nrhs * 12.0 * sizeof(T), s);
-    k_bicg_resume<T><<<dim3(grid1d(n), 1, nrhs), 256, 0, s>>>(rin, x, r, rh, p, v, partials, pstride, st, nactive, n);
+    k_bicg_resume<T><<<dim3(grid_vec(n, nrhs), 1, nrhs), 256, 0, s>>>(rin, x, r, rh, p, v, partials, pstride, st, nactive, n);
 }
 template void launch_bicg_resume<float>(const float*, float*, float*, float*, float*, float*, double*, int, RhsState*,
                                         int*, size_t, int, cudaStream_t);
@@ -706,7 +712,7 @@ template void launch_bicg_resume<double>(const double*, double*, double*, double
 template <typename T>
 __global__ void k_bicg_p(const T* __restrict__ r, T* __restrict__ p, const T* __restrict__ v, const RhsState* st,
                          size_t n) {
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!st[b].active) return;
@@ -727,13 +733,13 @@ __global__ void k_bicg_p(const T* __restrict__ r, T* __restrict__ p, const T* __
 template <typename T>
 void launch_bicg_p(const T* r, T* p, const T* v, const RhsState* st, size_t n, int nrhs, cudaStream_t s) {
     ProfScope prof(PK_BICG_P, (int)n, 1, (double)n * nrhs * 8.0 * sizeof(T), s);
-    launch_pdl(k_bicg_p<T>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, r, p, v, st, n);
+    launch_pdl(k_bicg_p<T>, dim3(grid_vec(n, nrhs), 1, nrhs), dim3(256), 0, s, r, p, v, st, n);
 }
 
 template <typename T>
 __global__ void k_bicg_s(const T* __restrict__ r, const T* __restrict__ v, T* __restrict__ sv, const RhsState* st,
                          size_t n) {
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!st[b].active) return;
@@ -749,7 +755,7 @@ __global__ void k_bicg_s(const T* __restrict__ r, const T* __restrict__ v, T* __
 template <typename T>
 void launch_bicg_s(const T* r, const T* v, T* sv, const RhsState* st, size_t n, int nrhs, cudaStream_t s) {
     ProfScope prof(PK_BICG_S, (int)n, 1, (double)n * nrhs * 6.0 * sizeof(T), s);
-    launch_pdl(k_bicg_s<T>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, r, v, sv, st, n);
+    launch_pdl(k_bicg_s<T>, dim3(grid_vec(n, nrhs), 1, nrhs), dim3(256), 0, s, r, v, sv, st, n);
 }
 
 // x += alpha p^ + omega s^, r = s - omega t and the sums for the next scalars. SAME: s^ is s itself (no
@@ -760,7 +766,7 @@ __global__ void __launch_bounds__(256) k_bicg_xr(T* x, const T* __restrict__ ph,
                                                  const T* __restrict__ rh, T* r, double* partials, int pstride,
                                                  RhsState* st, int* nactive, size_t n) {
     __shared__ double sh[96];
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!st[b].active) return;
@@ -823,7 +829,7 @@ void launch_bicg_xr(T* x, const T* ph, const T* shv, const T* sv, const T* t, co
                     int pstride, RhsState* st, int* nactive, size_t n, int nrhs, cudaStream_t s) {
     const bool same = shv == sv;
     ProfScope prof(PK_BICG_XR, (int)n, 1, (double)n * nrhs * (same ? 14.0 : 16.0) * sizeof(T), s);
-    launch_pdl(same ? k_bicg_xr<T, true> : k_bicg_xr<T, false>, dim3(grid1d(n), 1, nrhs), dim3(256), 0, s, x, ph, shv,
+    launch_pdl(same ? k_bicg_xr<T, true> : k_bicg_xr<T, false>, dim3(grid_vec(n, nrhs), 1, nrhs), dim3(256), 0, s, x, ph, shv,
                sv, t, rh, r, partials, pstride, st, nactive, n);
 }
 
@@ -989,7 +995,7 @@ __global__ void __launch_bounds__(NT) k_restrict_g(LevelDev Lf, LevelDev Lc, con
                                                    T wj, const T* __restrict__ f, const T* __restrict__ ec,
                                                    T* __restrict__ fc, const RhsState* st) {
     __shared__ RestrictTile<T, GRCX, GRCZ, NT> sm;
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int b = blockIdx.z;
     restrict_tile_stage<T, GRCX, GRCZ, NT>(sm, Lf, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);   // model data
     pdl_wait();
@@ -1003,7 +1009,7 @@ __global__ void __launch_bounds__(NT) k_prolong_g(LevelDev Lf, LevelDev Lc, cons
                                                          T b2, T wj, const T* __restrict__ f, const T* __restrict__ ec,
                                                          T* __restrict__ out, const RhsState* st, int accumulate) {
     __shared__ ProlongTile<T, GPX, GPZ, NT> sm;
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int b = blockIdx.z;
     prolong_tile_stage<T, GPX, GPZ, NT>(sm, Lf, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);   // model data
     pdl_wait();
@@ -1020,7 +1026,7 @@ __global__ void __launch_bounds__(NT) k_resid_restrict_g(LevelDev Lf, LevelDev L
                                                          T b2, T wj, const T* __restrict__ f, const T* __restrict__ e,
                                                          T* __restrict__ g, T* __restrict__ fc, const RhsState* st) {
     __shared__ ResidRestrictTile<T, GRCX, GRCZ, NT> sm;
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int b = blockIdx.z;
     resid_restrict_tile_stage<T, GRCX, GRCZ, NT>(sm, Lf, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);
     pdl_wait();
@@ -1087,7 +1093,7 @@ __global__ void __launch_bounds__(NT) k_prolong2_g(LevelDev Lf, LevelDev Lm, Lev
                                                           const T* __restrict__ ec, const T* em, T* out,
                                                           const RhsState* st, int acc_f, int acc_m) {
     __shared__ Prolong2Tile<T, GPX, GPZ, NT> sm;
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int b = blockIdx.z;
     prolong2_tile_stage<T, GPX, GPZ, NT>(sm, Lf, Lm, blockIdx.x, blockIdx.y, b, hwv[b], b1, b2, threadIdx.x);
     pdl_wait();
@@ -1233,7 +1239,7 @@ template <typename T> __device__ __forceinline__ cx<T> sh_dn(cx<T> a) {
 // holding u1 of three rows in registers and loading two rows ahead; the
 // neighbour columns across a lane boundary come by shuffle. r is zero outside
 // the grid. 320 right-hand sides of 441 x 241 in FP32: packed sums 57.3 -> 54.9 us, two steps per loop
-// (the rotating rows need no moves) -> 52 us.
+// (the rotating rows need no moves) at three blocks per SM -> 51 us (at the two that 90 registers leave 60).
 constexpr int RM_COLS = 30;   // coarse columns per warp
 
 // The marching loop; EDGE = false when every row and column the warp touches
@@ -1307,19 +1313,20 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_restrict(LevelDev Lf, LevelDev Lc, const T* __restrict__ w2, T b1, T b2,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_restrict(LevelDev Lf, LevelDev Lc, const T* __restrict__ w2, T b1, T b2,
                                                   T wj, const T* __restrict__ f, T* __restrict__ fc,
                                                   const RhsState* st, int ks) {
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!rhs_active(st, b)) return;
     const int lane = threadIdx.x & 31;
-    const int Ib = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RM_COLS - 1;   // coarse column of lane 0
-    if (Ib + 1 >= Lc.nx) return;   // uniform in the warp; the kernel has no block barrier
+    const int cw = (Lc.nx + RM_COLS - 1) / RM_COLS, wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int Ib = wid % cw * RM_COLS - 1;   // coarse column of lane 0
+    const int K0 = wid / cw * ks, K1 = min(K0 + ks, Lc.nz);
+    if (K0 >= Lc.nz) return;   // uniform in the warp; the kernel has no block barrier
     const int nx = Lf.nx, nz = Lf.nz;
     const int I = Ib + lane;
-    const int K0 = blockIdx.y * ks, K1 = min(K0 + ks, Lc.nz);
     const size_t nf = (size_t)nx * nz;
     const T* fb = f + 2 * nf * b;
     const T* m2 = static_cast<const T*>(Lf.m2) + (size_t)b * Lf.mstride;
@@ -1333,15 +1340,31 @@ __global__ void __launch_bounds__(256) k_restrict(LevelDev Lf, LevelDev Lc, cons
         restrict_march<T, false>(nx, nz, Lc.nx, 2 * I, I, lane, K0, K1, fb, m2, hw * b1, hw * b2, wj, fcb);
 }
 
-// Rows per block of the marching kernels: long segments amortise the rows
+// Rows per warp of the marching kernels. FP32: long segments amortise the rows
 // recomputed at segment ends; short ones give enough warps when the batch is
-// small (aim: 32 warps per SM on 152 SMs). FP64 issues an instruction in 16 cycles of an SM: 8 warps
-// keep its pipe busy, and more of them only add rows that are computed twice.
-template <typename T> constexpr unsigned kMarchWarps = sizeof(T) == 4 ? 32 : 8;
-inline int march_rows(int col_warps, int rows, int nrhs, int longest, unsigned warps) {
+// small (aim: 32 warps per SM on 152 SMs).
+// FP64: a quarter of an SM takes 64 cycles for an instruction of a warp, so the time is the warps of
+// the busiest quarter times a warp's rows, of which `lead` are recomputed: the least over the segment
+// lengths. (241 x 191, two right-hand sides: restriction 25 us at 4 coarse rows, 192 warps, 17 us at 2.)
+template <typename T>
+inline int march_rows(int col_warps, int rows, int nrhs, int longest, int step, int lead) {
     int zs = longest;
-    while (zs > 4 && (size_t)col_warps * ((rows + zs - 1) / zs) * nrhs < 152u * warps) zs /= 2;
+    if (sizeof(T) == 4) {
+        while (zs > 4 && (size_t)col_warps * ((rows + zs - 1) / zs) * nrhs < 152u * 32u) zs /= 2;
+        return zs;
+    }
+    size_t best = SIZE_MAX;
+    for (int k = longest; k >= step; k -= step) {
+        const size_t warps = (size_t)col_warps * ((rows + k - 1) / k) * nrhs;
+        const size_t cost = (warps + 4 * 152 - 1) / (4 * 152) * (k + lead);
+        if (cost < best) { best = cost; zs = k; }
+    }
     return zs;
+}
+// Warps per block of the marching kernels, whose warps (column strips of a row segment, then those of the
+// next) fill the blocks without gaps: as few as give every SM a block.
+inline int march_warps(int warps, int nrhs, int most) {
+    return (int)std::min<size_t>(most, ((size_t)warps * nrhs + 151) / 152);
 }
 
 template <typename T>
@@ -1356,9 +1379,10 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
                    s);
     if (Lf.m2 && !Lf.rho) {   // finest constant-density level; a density level is stored like a coarse one
         const int cw = (Lc.nx + RM_COLS - 1) / RM_COLS;
-        const int ks = march_rows(cw, Lc.nz, nrhs, 16, kMarchWarps<T>);
-        dim3 grd((cw + 7) / 8, (Lc.nz + ks - 1) / ks, nrhs);
-        launch_pdl(k_restrict<T>, grd, dim3(256), 0, s, Lf, Lc, w2, (T)b1, (T)b2, (T)wj, f, fc, st, ks);
+        const int ks = march_rows<T>(cw, Lc.nz, nrhs, 16, 1, 2);
+        const int nw = cw * ((Lc.nz + ks - 1) / ks), wb = march_warps(nw, nrhs, 8);
+        dim3 grd((nw + wb - 1) / wb, 1, nrhs);
+        launch_pdl(k_restrict<T>, grd, dim3(32 * wb), 0, s, Lf, Lc, w2, (T)b1, (T)b2, (T)wj, f, fc, st, ks);
     } else {
         launch_restrict_g<T, false>(tile, Lf, Lc, w2, b1, b2, wj, f, (const T*)nullptr, fc, st, nrhs, s);
     }
@@ -1382,7 +1406,7 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
 // the cycles, waiting for loads otherwise. The damping terms only where a row or the warp's columns have
 // any, and packed sums: 142 -> 128 us. A cap of 128 registers for mode 1 spills (137 us). FP64 is bound
 // by its arithmetic at two results per clock and SM: the first step's unused u3, the rows above
-// the segment and the second divide of odd rows left out, and longer segments (march_rows): 80 -> 61 us on 241 x
+// the segment and the second divide of odd rows left out, blocks without idle warps: 80 -> 39 us on 241 x
 // 191 with two right-hand sides. In FP32 the skipped rows cost more in scheduling than they save (156 us).
 constexpr int PM_COLS = 60;   // fine output columns per warp
 
@@ -1556,7 +1580,7 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
     }
 }
 
-constexpr int PM_WARPS = 4;   // warps per block of the marching prolongation
+constexpr int PM_WARPS = 4;   // most warps per block of the marching prolongation
 
 template <typename T, int MODE>
 __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev Lc, int npml, T acoef,
@@ -1565,14 +1589,15 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
                                                  T* __restrict__ out, T* __restrict__ y, const T* __restrict__ aux,
                                                  double* partials, int pstride, RhsState* st, int accumulate, int zs) {
     __shared__ double shred[96];
-    pdl_trigger();
+    pdl_trigger_for<T>();
     pdl_wait();
     const int b = blockIdx.z;
     if (!rhs_active(st, b)) return;   // uniform in the block
     const int lane = threadIdx.x & 31;
     const int nx = Lf.nx, nz = Lf.nz, cnx = Lc.nx, cnz = Lc.nz;
-    const int Jb = (blockIdx.x * PM_WARPS + (threadIdx.x >> 5)) * (PM_COLS / 2) - 1;   // coarse column of lane 0
-    const int Z0 = blockIdx.y * zs, Z1 = min(Z0 + zs, nz);
+    const int cw = (nx + PM_COLS - 1) / PM_COLS, wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int Jb = wid % cw * (PM_COLS / 2) - 1;   // coarse column of lane 0
+    const int Z0 = wid / cw * zs, Z1 = min(Z0 + zs, nz);
     const size_t nf = (size_t)nx * nz, nc = (size_t)cnx * cnz;
     const T* fb = f + 2 * nf * b;
     const T* eb = ec + 2 * nc * b;
@@ -1582,7 +1607,7 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
     T* yb = y + 2 * nf * b;
     const T hw = w2[b];
     T d0 = 0, d1 = 0, d2 = 0;
-    if (2 * (Jb + 1) < nx) {   // the warp has output columns (uniform in the warp)
+    if (Z0 < nz) {   // the warp has output rows (uniform in the warp)
         // fine columns 2 Jb .. 2 Jb + 63, coarse columns Jb .. Jb + 31 and rows
         // Z0 - 4 .. Z1 + 3 (coarse rows Z0/2 - 2 .. Z1/2 + 2) inside the grid?
         const bool edge = Jb < 0 || 2 * Jb + 63 >= nx || Jb + 31 >= cnx || Z0 < 4 || Z1 + 3 >= nz ||
@@ -1598,8 +1623,8 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
     else {
         const T vv[3] = {d0, d1, d2};
         double acc[3];
-        const int nblk = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
-        if (last_block_reduce_t<3, T>(vv, acc, shred, partials + (size_t)b * pstride, nblk, blk, &st[b].counter[3])) {
+        if (last_block_reduce_t<3, T>(vv, acc, shred, partials + (size_t)b * pstride, gridDim.x, blockIdx.x,
+                                      &st[b].counter[3])) {
             if (threadIdx.x == 0) {
                 RhsState& S = st[b];
                 if (MODE == 1) {   // alpha = rho / <rh, v>
@@ -1623,10 +1648,13 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
 }
 
 // Grid of the marching prolongation for a fine level of nx x nz nodes.
-inline dim3 prolong_grid(int nx, int nz, int nrhs, int longest, unsigned warps, int* zs) {
+template <typename T>
+inline dim3 prolong_grid(int nx, int nz, int nrhs, int longest, int* zs, int* block) {
     const int cw = (nx + PM_COLS - 1) / PM_COLS;
-    *zs = march_rows(cw, nz, nrhs, longest, warps);
-    return dim3((cw + PM_WARPS - 1) / PM_WARPS, (nz + *zs - 1) / *zs, nrhs);
+    *zs = march_rows<T>(cw, nz, nrhs, longest, 4, 4);   // at least 4 rows: the partial sums' bound
+    const int nw = cw * ((nz + *zs - 1) / *zs), wb = march_warps(nw, nrhs, PM_WARPS);
+    *block = 32 * wb;
+    return dim3((nw + wb - 1) / wb, 1, nrhs);
 }
 
 template <typename T>
@@ -1650,19 +1678,19 @@ void launch_prolong(int mode, const LevelDev& Lf, const LevelDev& Lc, int npml, 
         return;
     }
     // finest level: the tile choice is the longest row segment (16 or 32 rows)
-    int zs = 0;
-    const dim3 grd = prolong_grid(Lf.nx, Lf.nz, nrhs, tile == 0 ? 16 : 32, kMarchWarps<T>, &zs);
+    int zs = 0, block = 0;
+    const dim3 grd = prolong_grid<T>(Lf.nx, Lf.nz, nrhs, tile == 0 ? 16 : 32, &zs, &block);
     if (mode == 0)
-        launch_pdl(k_prolong<T, 0>, grd, dim3(32 * PM_WARPS), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
+        launch_pdl(k_prolong<T, 0>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
     else if (mode == 1)
-        launch_pdl(k_prolong<T, 1>, grd, dim3(32 * PM_WARPS), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
+        launch_pdl(k_prolong<T, 1>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
     else if (mode == 2)
-        launch_pdl(k_prolong<T, 2>, grd, dim3(32 * PM_WARPS), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
+        launch_pdl(k_prolong<T, 2>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
     else
-        launch_pdl(k_prolong<T, 3>, grd, dim3(32 * PM_WARPS), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
+        launch_pdl(k_prolong<T, 3>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
 }
 
@@ -1877,7 +1905,7 @@ __device__ __forceinline__ int tail_row(int p, float rnx) { return (int)(((float
 template <typename T>
 __global__ void __launch_bounds__(1024, 1) k_tail(const __grid_constant__ TailArgs a, const RhsState* st) {
     extern __shared__ __align__(16) unsigned char tail_smem[];
-    pdl_trigger();
+    pdl_trigger_for<T>();
     const int b = blockIdx.x;
     const T hw = (T)a.w2[b], b1 = (T)a.b1, b2 = (T)a.b2, wj = (T)a.wj;
     const T hb1 = hw * b1, hb2 = hw * b2;
