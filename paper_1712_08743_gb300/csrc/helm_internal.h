@@ -183,8 +183,8 @@ class NvtxRange {
 enum ProfKernel : int {
     PK_APPLY, PK_APPLY_DOTS, PK_RESID64, PK_REFINE, PK_BICG_INIT, PK_BICG_RESUME, PK_BICG_P, PK_BICG_S, PK_BICG_XR,
     PK_RESTRICT, PK_PROLONG, PK_RESTRICT_G, PK_CORRECT_RESTRICT, PK_RESID_RESTRICT, PK_PROLONG_G, PK_PROLONG2_G, PK_TAIL, PK_COARSE_DENSE,
-    PK_DENSE_INVERT, PK_COARSE_INVERT, PK_FG_NORM, PK_FG_SCALE, PK_FG_DOTS, PK_FG_AXPY, PK_FG_FINISH,
-    PK_FG_BACKSOLVE, PK_FG_UPDATE, PK_FCYCLE, PK_OTHER, PK_COUNT
+    PK_DENSE_INVERT, PK_COARSE_INVERT, PK_FG_SCALE, PK_FG_DOTS, PK_FG_AXPY, PK_FG_FINISH,
+    PK_FG_UPDATE, PK_FCYCLE, PK_OTHER, PK_COUNT
 };
 bool prof_on();
 class ProfScope {

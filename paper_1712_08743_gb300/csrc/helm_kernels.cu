@@ -1300,7 +1300,7 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
         const cx<T> h0 = hsum(r0, r1), h1 = hsum(s0, s1);
         if (K > K0) {
             acc = padd(acc, h0);   // completes coarse row K - 1
-            if (wr) stc(fcb, (size_t)(K - 1) * cnx + I, T(0.25) * acc);
+            if (wr) stc(fcb, (K - 1) * cnx + I, T(0.25) * acc);
         }
         acc = pfma(T(2), h1, h0);
         ua0 = uc0; ua1 = uc1; ub0 = ud0; ub1 = ud1;
@@ -1309,7 +1309,7 @@ __device__ __forceinline__ void restrict_march(int nx, int nz, int cnx, int c0, 
     cx<T> r0, r1;
     resid(2 * K1, B, ua0, ua1, ub0, ub1, u1of(C.f0, C.m0), u1of(C.f1, C.m1), r0, r1);
     acc = acc + hsum(r0, r1);
-    if (wr) stc(fcb, (size_t)(K1 - 1) * cnx + I, T(0.25) * acc);
+    if (wr) stc(fcb, (K1 - 1) * cnx + I, T(0.25) * acc);
 }
 
 template <typename T>
@@ -1932,7 +1932,7 @@ __global__ void __launch_bounds__(1024, 1) k_tail(const __grid_constant__ TailAr
     const int nL = a.lv[a.L].nx * a.lv[a.L].nz;
     const T* Mg = static_cast<const T*>(a.minv) + 2 * (size_t)nL * nL * a.slot[b];
     cx<T>* Ms = base + a.minv_off;
-    // the inverse is written by k_coarse_invert before the first ordinary launch of the solve
+    // the inverse is written before the first ordinary launch of the solve
     if (a.minv_smem)
         for (int t = tid; t < nL * nL; t += nth) Ms[t] = ldc(Mg, t);
     pdl_wait();   // the coefficients above are model data; everything below depends on earlier kernels

@@ -52,3 +52,24 @@ def test_residual_at_both_sides_of_the_line(hg, precision, density, tol, below):
         assert np.linalg.norm(res) <= tol * (1 + 1e-3) * np.linalg.norm(f[k]), k
     model.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("coarse", ["DENSE", "FUSED"])
+def test_few_large_right_hand_sides(hg, coarse):
+    """Four right-hand sides of 724 x 726: the dense end and the persistent cycle, which the last V takes too."""
+    px, pz, nrhs = 708, 710, 4
+    assert 8 * (px + 2 * NPML) * (pz + 2 * NPML) * nrhs >= 16 << 20
+    rng = np.random.default_rng(3)
+    c = models.layered_model(rng, px, pz, 10.0, 6, 1500.0, 3500.0)
+    ctx = hg.Context(0)
+    model = hg.helm_create_model(ctx, 1.0 / c, 10.0, NPML, 0.5)
+    om = 2 * np.pi * np.linspace(3.0, 5.0, nrhs)
+    f = models.random_complex(rng, (nrhs, pz + 2 * NPML, px + 2 * NPML), np.complex64).astype(np.complex128)
+    u, st, rc = hg.helm_solve(model, om, f=f, opts=dict(tol=1e-8, coarse=getattr(hg, "HELM_COARSE_" + coarse)))
+    assert rc == hg.HELM_OK and all(s["converged"] for s in st)
+    alpha = hz.damping_profile(px, pz, NPML, 0.5)
+    B = hz.operator(oracle.pad_slowness(1.0 / c, NPML), 10.0, om[-1], alpha)
+    res = f[-1].ravel() - B @ u[-1].ravel()
+    assert np.linalg.norm(res) <= 1e-8 * (1 + 1e-3) * np.linalg.norm(f[-1])
+    model.close()
+    ctx.close()
