@@ -397,6 +397,8 @@ __global__ void __launch_bounds__(256) k_dense_mirror(TriShape sh, T* minv) {
     }
 }
 
+__global__ void k_order() {}
+
 // e_b (+)= M_d^-1 f_b for the right-hand sides of one group (consecutive RHS of
 // one slot, group g = [grp[g], grp[g+1])); one warp per row of the inverse, the
 // row held in registers (NR complex values per lane) and reused for
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(256) k_coarse_dense(int n, const T* __restrict
     const T* Mr = minv + 2 * ((size_t)slot[b0] * n * n + (size_t)min(row, n - 1) * n);
     static_assert(32 * NR >= kDenseMaxPoints, "a row of the inverse in one warp's registers");
     cx<T> rv[NR];
-    // this warp's row is model data: load it before waiting on the previous kernel
+    // this warp's row is ordered before any early launch (launch_order): load it ahead of the wait
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
         const int j = lane + 32 * k;
@@ -487,6 +489,11 @@ bool dense_invert_fits(int nx, int nz) {
     return nx * nz <= kDenseMaxPoints && std::min(nx, nz) <= kTriMaxW && std::max(nx, nz) >= kTriMinBlocks;
 }
 
+void launch_order(cudaStream_t s) {
+    k_order<<<1, 32, 0, s>>>();
+    count_launches(1);
+}
+
 template <typename T, int RT>
 static void dense_invert_rt(const TriShape& sh, const double* gk, size_t gks, const double* w2s, const int* mods,
                             int nslots, double b1, double b2, T* minv, int* err, cudaStream_t s) {
@@ -505,7 +512,7 @@ static void dense_invert_rt(const TriShape& sh, const double* gk, size_t gks, co
 // case, and a pivot's work grows with the square of the block.
 template <typename T>
 cudaError_t launch_dense_invert(const LevelDev& Ld, const double* w2s, const int* mods, int nslots, double b1,
-                                double b2, T* minv, int* err, cudaStream_t s) {
+                                double b2, T* minv, int* err, cudaStream_t s, bool order) {
     cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     const double n = (double)Ld.nx * Ld.nz;
@@ -520,12 +527,13 @@ cudaError_t launch_dense_invert(const LevelDev& Ld, const double* w2s, const int
     if (sh.w <= 16) dense_invert_rt<T, 1>(sh, gk, Ld.gkstride, w2s, mods, nslots, b1, b2, minv, err, s);
     else if (sh.w <= 32) dense_invert_rt<T, 2>(sh, gk, Ld.gkstride, w2s, mods, nslots, b1, b2, minv, err, s);
     else dense_invert_rt<T, 3>(sh, gk, Ld.gkstride, w2s, mods, nslots, b1, b2, minv, err, s);
+    if (order) launch_order(s);
     return cudaGetLastError();
 }
 template cudaError_t launch_dense_invert<float>(const LevelDev&, const double*, const int*, int, double, double,
-                                                float*, int*, cudaStream_t);
+                                                float*, int*, cudaStream_t, bool);
 template cudaError_t launch_dense_invert<double>(const LevelDev&, const double*, const int*, int, double, double,
-                                                 double*, int*, cudaStream_t);
+                                                 double*, int*, cudaStream_t, bool);
 
 template <typename T>
 void launch_coarse_dense(int n, const T* minv, const int* slot, const int* grp, int ngroups, int maxg, const T* f,

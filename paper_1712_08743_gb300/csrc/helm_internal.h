@@ -145,8 +145,8 @@ struct DBuf {
 };
 
 // Launch with programmatic stream serialization (the kernel must call pdl_wait
-// before reading anything an earlier kernel of the stream writes), which hides a launch
-// and the first loads of a kernel that takes a few microseconds. A grid of more than two full GPUs of
+// before reading anything an earlier kernel of the stream writes; what launch_order has ordered
+// may be read before it), which hides a launch and the first loads of a kernel that takes a few microseconds. A grid of more than two full GPUs of
 // threads starts when the kernel before has ended: early, its blocks only take room and L2 from that
 // one (320 right-hand sides of 441 x 241: 273 -> 262 ms, 128: 234 -> 223 ms; a line at one GPU: 265 ms, as
 // it takes the 320 blocks of the tail too; none for any grid: one right-hand side of 1041 x 1041 209 -> 221 ms).
@@ -348,11 +348,17 @@ template <typename T>
 void launch_coarse(int n, const T* minv, const int* slot, const T* fL, T* eL, const RhsState* st,
                    int nrhs, cudaStream_t s);
 // Dense exact solve of one coarse level (helm_dense.cu): whether a level can be inverted, and
-// the inverses of all slots into minv [nslots][n][n] (no workspace).
+// the inverses of all slots into minv [nslots][n][n] (no workspace). The launchers that form an
+// inverse end with launch_order: every later kernel of the stream may read it before its pdl_wait.
 bool dense_invert_fits(int nx, int nz);
+// An empty kernel launched the ordinary way: it starts when everything before it in the stream has ended
+// with its writes visible, and a kernel launched early behind it starts no sooner than it ends. Without it
+// the chain of early launches that follows an inversion orders its loads ahead of pdl_wait after the
+// inversion's last blocks' exits only, not after their writes.
+void launch_order(cudaStream_t s);
 template <typename T>
 cudaError_t launch_dense_invert(const LevelDev& Ld, const double* w2s, const int* mods, int nslots, double b1,
-                                double b2, T* minv, int* err, cudaStream_t s);
+                                double b2, T* minv, int* err, cudaStream_t s, bool order = true);
 // e (+)= M_d^-1 f per right-hand side; grp: [ngroups + 1] boundaries of groups of
 // at most maxg (<= 8) consecutive right-hand sides sharing a slot.
 template <typename T>

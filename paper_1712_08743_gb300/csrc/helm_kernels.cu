@@ -1853,7 +1853,7 @@ void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int*
     if (std::fabs(b2) >= 0.1 * std::fabs(b1) && b2 != 0.0 && dense_invert_fits(Lc.nx, Lc.nz)) {
         err = reinterpret_cast<int*>(work + nn * 2 * nslots - 1);   // a flag in the workspace's last element
         if (launch_dense_invert<double>(Lc, w2_slots, mod_slots, nslots, b1, b2,
-                                        reinterpret_cast<double*>(minv_d), err, s) == cudaSuccess)
+                                        reinterpret_cast<double*>(minv_d), err, s, false) == cudaSuccess)
             launch_cast_complex<float>(reinterpret_cast<const double*>(minv_d), reinterpret_cast<float*>(minv_f),
                                        nn * nslots, s);
         else
@@ -1863,6 +1863,7 @@ void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int*
     k_coarse_invert<<<nslots, 1024, 0, s>>>(Lc.nx, Lc.nz, static_cast<const double*>(Lc.gk),
                                             kGalerkinCoefs * n, w2_slots, mod_slots, b1, b2, work, minv_f, minv_d,
                                             err);
+    launch_order(s);   // the tail reads the inverse ahead of its wait
 }
 
 // ================================================================ tail
@@ -1932,7 +1933,7 @@ __global__ void __launch_bounds__(1024, 1) k_tail(const __grid_constant__ TailAr
     const int nL = a.lv[a.L].nx * a.lv[a.L].nz;
     const T* Mg = static_cast<const T*>(a.minv) + 2 * (size_t)nL * nL * a.slot[b];
     cx<T>* Ms = base + a.minv_off;
-    // the inverse is written before the first ordinary launch of the solve
+    // the inverse is ordered before any early launch (launch_order)
     if (a.minv_smem)
         for (int t = tid; t < nL * nL; t += nth) Ms[t] = ldc(Mg, t);
     pdl_wait();   // the coefficients above are model data; everything below depends on earlier kernels
