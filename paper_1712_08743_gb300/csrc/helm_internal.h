@@ -365,9 +365,10 @@ template <typename T>
 void launch_coarse_dense(int n, const T* minv, const int* slot, const int* grp, int ngroups, int maxg, const T* f,
                          T* e, int accumulate, const RhsState* st, cudaStream_t s);
 // Inverses of the tail's coarsest level in FP64 (minv_d) and rounded to FP32 (minv_f).
-// work: [nslots][n][2n] double2.
+// work: [nslots][n][2n] double2; err: one int, apart from work (the pivoted kernel reads it while it writes work).
 void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int* mod_slots, int nslots,
-                          double b1, double b2, double2* work, float2* minv_f, double2* minv_d, cudaStream_t s);
+                          double b1, double b2, double2* work, int* err, float2* minv_f, double2* minv_d,
+                          cudaStream_t s);
 
 // Persistent F-cycle (helm_fcycle.cu): the steps of one cycle from level ls down
 // to the dense level, in one cooperative launch. Step: type | FC_ACC (add to the

@@ -1847,22 +1847,21 @@ __global__ void __launch_bounds__(1024) k_coarse_invert(int nx, int nz, const do
 // with a serial search per column, took 2560 us. The pivoted kernel is launched behind it and
 // returns at once unless the elimination reported a pivot.
 void launch_coarse_invert(const LevelDev& Lc, const double* w2_slots, const int* mod_slots, int nslots, double b1,
-                          double b2, double2* work, float2* minv_f, double2* minv_d, cudaStream_t s) {
+                          double b2, double2* work, int* err, float2* minv_f, double2* minv_d, cudaStream_t s) {
     const size_t n = (size_t)Lc.nx * Lc.nz, nn = n * n;
-    int* err = nullptr;
+    const int* need = nullptr;
     if (std::fabs(b2) >= 0.1 * std::fabs(b1) && b2 != 0.0 && dense_invert_fits(Lc.nx, Lc.nz)) {
-        err = reinterpret_cast<int*>(work + nn * 2 * nslots - 1);   // a flag in the workspace's last element
         if (launch_dense_invert<double>(Lc, w2_slots, mod_slots, nslots, b1, b2,
-                                        reinterpret_cast<double*>(minv_d), err, s, false) == cudaSuccess)
+                                        reinterpret_cast<double*>(minv_d), err, s, false) == cudaSuccess) {
             launch_cast_complex<float>(reinterpret_cast<const double*>(minv_d), reinterpret_cast<float*>(minv_f),
                                        nn * nslots, s);
-        else
-            err = nullptr;
+            need = err;
+        }
     }
     ProfScope prof(PK_COARSE_INVERT, Lc.nx, Lc.nz, (double)nn * nslots * 24.0, s);
     k_coarse_invert<<<nslots, 1024, 0, s>>>(Lc.nx, Lc.nz, static_cast<const double*>(Lc.gk),
                                             kGalerkinCoefs * n, w2_slots, mod_slots, b1, b2, work, minv_f, minv_d,
-                                            err);
+                                            need);
     launch_order(s);   // the tail reads the inverse ahead of its wait
 }
 

@@ -27,7 +27,8 @@ constexpr int kNoAllocCoarse = HELM_COARSE_AUTO;   // the coarse end helm_vcycle
 
 // The scratch area. In host code `g_noalloc_scratch` names a host-side stand-in,
 // not device memory: kernels get the device address from cudaGetSymbolAddress.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+// the area that calls carve up, and one int behind it: the tail's elimination flag
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + sizeof(int)];
 
 std::mutex g_mu;
 void* g_base[kMaxDevices] = {nullptr};
@@ -126,6 +127,7 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
             p.work = take(sizeof(double2) * nc * nc * 2 * nslots);
             p.minv = take(sizeof(float2) * nc * nc * nslots);
             p.md = take(sizeof(double2) * nc * nc * nslots);
+            p.err = kNoAllocScratchBytes;
             p.top = m->lt[0];
         }
         for (int l = 1; l <= p.top; ++l) {
@@ -185,8 +187,8 @@ extern "C" int helm_vcycle_noalloc(helm_model* m, int nrhs, const double* omega,
         if (!use_dense)
             launch_coarse_invert(level_dev(m, L, true), reinterpret_cast<const double*>(base + o_w2s),
                                  reinterpret_cast<const int*>(base + o_mods), nslots, beta1, beta2,
-                                 reinterpret_cast<double2*>(base + plan.work), reinterpret_cast<float2*>(base + plan.minv),
-                                 reinterpret_cast<double2*>(base + plan.md), s);
+                                 reinterpret_cast<double2*>(base + plan.work), reinterpret_cast<int*>(base + plan.err),
+                                 reinterpret_cast<float2*>(base + plan.minv), reinterpret_cast<double2*>(base + plan.md), s);
         MgCall mc;
         mc.w2 = dw2;
         mc.w2f = reinterpret_cast<const float*>(base + o_w2f);

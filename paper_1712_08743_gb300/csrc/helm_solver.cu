@@ -726,7 +726,7 @@ static int fgmres_inner(const SolveCtx& c, Inner<T>& w, FgBufs<T>& f, const T* r
 // copies). One inverse per distinct (model, frequency) pair: slot[b].
 struct CoarseSet {
     DBuf work, mf, md;
-    DBuf err;                          // dense path: set by the inversion (coarse_failed)
+    DBuf err;                          // set by the inversion: dense path, see coarse_failed; tail, the pivoted kernel reads it
     Upload up;                         // slot, w2s, mods and (dense path) grp
     const int* slot = nullptr;
     const int* grp = nullptr;
@@ -801,12 +801,13 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
     TRY_ALLOC(cs.work, sizeof(double2) * nn * 2 * cs.nslots, s);
     TRY_ALLOC(cs.mf, sizeof(float2) * nn * cs.nslots, s);
     TRY_ALLOC(cs.md, sizeof(double2) * nn * cs.nslots, s);
+    if (!cs.err.p) TRY_ALLOC(cs.err, sizeof(int), s);
     const size_t o_slot = cs.up.add(slot), o_w2s = cs.up.add(w2s), o_mods = cs.up.add(mods);
     TRY_SEND(cs.up, s);
     cs.slot = cs.up.at<int>(o_slot);
     count_launches(1);
     launch_coarse_invert(level_dev(m, (int)m->lv.size() - 1, true), cs.up.at<double>(o_w2s), cs.up.at<int>(o_mods),
-                         cs.nslots, b1, b2, cs.work.as<double2>(), cs.mf.as<float2>(), cs.md.as<double2>(), s);
+                         cs.nslots, b1, b2, cs.work.as<double2>(), cs.err.as<int>(), cs.mf.as<float2>(), cs.md.as<double2>(), s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }

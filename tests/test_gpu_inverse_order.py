@@ -63,7 +63,7 @@ int main() {
     return a ? 10 + a : b ? 20 + b : 0;
 }
 """.replace("TAIL_OR_DENSE", """if (tail)
-        launch_coarse_invert(L, w2, i, 1, 1.0, 0.5, (double2*)d, (float2*)d, (double2*)d, s);
+        launch_coarse_invert(L, w2, i, 1, 1.0, 0.5, (double2*)d, i, (float2*)d, (double2*)d, s);
     else
         launch_dense_invert<float>(L, w2, i, 1, 1.0, 0.5, (float*)d, i, s);""")
 
