@@ -28,6 +28,21 @@ class DeviceGuard {   // makes the context's device current for the call
     int prev_ = 0;
 };
 
+// Every call returns with its stream idle, on errors too: cudaFree of pool memory (a model's, a misfit
+// state's) takes all accesses to be over, and workspaces go back to a pool that other streams draw from.
+class Drain {
+  public:
+    explicit Drain(cudaStream_t s) : s_(s) {}
+    Drain(const Drain&) = delete;
+    Drain& operator=(const Drain&) = delete;
+    cudaError_t wait() { idle_ = true; return cudaStreamSynchronize(s_); }   // the end of a call that went well
+    ~Drain() { if (!idle_) cudaStreamSynchronize(s_); }
+
+  private:
+    cudaStream_t s_;
+    bool idle_ = false;
+};
+
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
 
 int check_opts(const helm_solve_opts& o) {
@@ -121,6 +136,7 @@ int create_model(helm_ctx* ctx, cudaStream_t s, int Px, int Pz, double h, const 
     auto fail = [&](cudaError_t e) {
         set_last_error(cudaGetErrorString(e));
         cudaGetLastError();
+        cudaStreamSynchronize(s);   // kernels that fill the model may be under way
         helm_destroy_model(m);
         return e == cudaErrorMemoryAllocation ? HELM_E_NOMEM : HELM_E_CUDA;
     };
@@ -281,7 +297,7 @@ int helm_create_model_rho(helm_ctx* ctx, int Px, int Pz, double h, const double*
 void helm_destroy_model(helm_model* m) {
     if (!m) return;
     DeviceGuard g(m->ctx->device);
-    if (m->slab) cudaFree(m->slab);   // waits for the work that uses it; the memory returns to the context's pool
+    if (m->slab) cudaFree(m->slab);   // no call leaves work on it behind (Drain); the memory returns to the context's pool
     delete m;
 }
 
@@ -315,6 +331,7 @@ int helm_solve(helm_model* m, int nrhs, const double* omega, const int* src_ix, 
     }
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t n = m->n();
     const size_t fbytes = sizeof(double) * 2 * n * nrhs;
     DBuf f64, u64, dsrc, fin;
@@ -347,7 +364,7 @@ int helm_solve(helm_model* m, int nrhs, const double* omega, const int* src_ix, 
     if (!o.device_ptrs) {
         HELM_CUDA_TRY(cudaMemcpyAsync(u_out, u_dev, fbytes, cudaMemcpyDeviceToHost, s));
     }
-    HELM_CUDA_TRY(cudaStreamSynchronize(s));
+    HELM_CUDA_TRY(drain.wait());
     return rc;
 }
 
@@ -361,6 +378,7 @@ int helm_apply(helm_model* m, int nrhs, const double* omega, int precision, cons
     }
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const bool dbl = precision == HELM_PREC_FP64;
     const size_t bytes = (dbl ? 16 : 8) * m->n() * nrhs;
     DBuf dw2, du, dy;
@@ -388,19 +406,21 @@ int helm_apply(helm_model* m, int nrhs, const double* omega, int precision, cons
                             static_cast<const float*>(up), static_cast<float*>(yp), (float)sc, nrhs, s);
     HELM_CUDA_TRY(cudaGetLastError());
     if (!device_ptrs) HELM_CUDA_TRY(cudaMemcpyAsync(y, yp, bytes, cudaMemcpyDeviceToHost, s));
-    HELM_CUDA_TRY(cudaStreamSynchronize(s));   // the host copies above are sources of async copies
+    HELM_CUDA_TRY(drain.wait());   // the host copies above are sources of async copies
     return HELM_OK;
 }
 
 int helm_time_kernel(helm_model* m, int kernel, int nrhs, double omega, int reps, double* ms, double* bytes) {
     if (!m || nrhs < 1 || reps < 1 || !finite_pos(omega) || !ms || !bytes) return HELM_E_INVALID;
     DeviceGuard g(m->ctx->device);
+    Drain drain(m->ctx->stream);
     return time_kernel(m, m->ctx->stream, kernel, nrhs, m->h * m->h * omega * omega, reps, ms, bytes);
 }
 
 int helm_autotune(helm_model* m, int nrhs, double omega, int* tiles_out) {
     if (!m || nrhs < 1 || !finite_pos(omega)) return HELM_E_INVALID;
     DeviceGuard g(m->ctx->device);
+    Drain drain(m->ctx->stream);
     int tiles[2 * kMaxLevels];
     int rc = autotune(m, m->ctx->stream, nrhs, m->h * m->h * omega * omega, 5, tiles);
     if (rc == HELM_OK && tiles_out) std::memcpy(tiles_out, tiles, sizeof(tiles));
@@ -433,6 +453,7 @@ int vcycle_call(helm_model* m, int nrhs, const double* omega, double beta1, doub
     }
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t bytes = 8 * m->n() * nrhs;
     DBuf dr, dz;
     const void* rp = r;
@@ -450,7 +471,7 @@ int vcycle_call(helm_model* m, int nrhs, const double* omega, double beta1, doub
                          static_cast<float*>(zp));
     if (rc != HELM_OK) return rc;
     if (!device_ptrs) HELM_CUDA_TRY(cudaMemcpyAsync(z, zp, bytes, cudaMemcpyDeviceToHost, s));
-    HELM_CUDA_TRY(cudaStreamSynchronize(s));
+    HELM_CUDA_TRY(drain.wait());
     return HELM_OK;
 }
 }  // namespace
@@ -495,6 +516,7 @@ int helm_fwi_forward(helm_model* m, int nfreq, const double* omega, int nshot, c
     }
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t dbytes = sizeof(double) * 2 * (size_t)nfreq * nshot * nrec;
     DBuf dobs, dcal;
     const double* dobs_p = static_cast<const double*>(d_obs);
@@ -514,7 +536,7 @@ int helm_fwi_forward(helm_model* m, int nfreq, const double* omega, int nshot, c
     if (rc != HELM_OK && rc != HELM_E_NOT_CONVERGED) { fwi_free(st); return rc; }
     if (!o.device_ptrs && d_cal_out) {
         cudaError_t e = cudaMemcpyAsync(d_cal_out, dcal_p, dbytes, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = drain.wait();
         if (e != cudaSuccess) { fwi_free(st); set_last_error(cudaGetErrorString(e)); return HELM_E_CUDA; }
     }
     helm_fwi_state* out = new helm_fwi_state();
@@ -533,6 +555,7 @@ int helm_fwi_backward(helm_fwi_state* state, double* grad_out, const helm_solve_
     helm_model* m = state->m;
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t gbytes = sizeof(double) * (size_t)m->Px * m->Pz;
     DBuf dgrad;
     double* grad_p = grad_out;
@@ -544,7 +567,7 @@ int helm_fwi_backward(helm_fwi_state* state, double* grad_out, const helm_solve_
     if (rc != HELM_OK && rc != HELM_E_NOT_CONVERGED) return rc;
     if (!o.device_ptrs) {
         HELM_CUDA_TRY(cudaMemcpyAsync(grad_out, grad_p, gbytes, cudaMemcpyDeviceToHost, s));
-        HELM_CUDA_TRY(cudaStreamSynchronize(s));
+        HELM_CUDA_TRY(drain.wait());
     }
     return rc;
 }
@@ -558,6 +581,7 @@ int helm_gn_hvp(helm_fwi_state* state, const double* dm, double* hdm_out, const 
     helm_model* m = state->m;
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t bytes = sizeof(double) * (size_t)m->Px * m->Pz;
     DBuf ddm, dh;
     const double* dm_p = dm;
@@ -575,7 +599,7 @@ int helm_gn_hvp(helm_fwi_state* state, const double* dm, double* hdm_out, const 
     if (rc != HELM_OK && rc != HELM_E_NOT_CONVERGED) return rc;
     if (!o.device_ptrs) {
         HELM_CUDA_TRY(cudaMemcpyAsync(hdm_out, h_p, bytes, cudaMemcpyDeviceToHost, s));
-        HELM_CUDA_TRY(cudaStreamSynchronize(s));
+        HELM_CUDA_TRY(drain.wait());
     }
     return rc;
 }
@@ -593,6 +617,7 @@ int helm_gn_step(helm_fwi_state* state, const double* grad, int cg_iters, double
     helm_model* m = state->m;
     DeviceGuard g(m->ctx->device);
     cudaStream_t s = m->ctx->stream;
+    Drain drain(s);
     const size_t bytes = sizeof(double) * (size_t)m->Px * m->Pz;
     DBuf dgrad, ddm;
     const double* g_p = grad;
@@ -611,7 +636,7 @@ int helm_gn_step(helm_fwi_state* state, const double* grad, int cg_iters, double
     if (rc != HELM_OK && rc != HELM_E_NOT_CONVERGED) return rc;
     if (!o.device_ptrs) {
         HELM_CUDA_TRY(cudaMemcpyAsync(dm_out, dm_p, bytes, cudaMemcpyDeviceToHost, s));
-        HELM_CUDA_TRY(cudaStreamSynchronize(s));
+        HELM_CUDA_TRY(drain.wait());
     }
     if (cg_rel_out) std::memcpy(cg_rel_out, rel.data(), sizeof(double) * rel.size());
     return rc;

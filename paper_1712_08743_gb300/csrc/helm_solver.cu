@@ -1504,7 +1504,7 @@ int gn_step(FwiState* st, cudaStream_t s, const double* g_dev, int iters, double
     return status;
 }
 
-void fwi_free(FwiState* st) {
+void fwi_free(FwiState* st) {   // no work on it is under way: every call returns with its stream idle
     if (!st) return;
     if (st->u64) cudaFree(st->u64);
     if (st->resid) cudaFree(st->resid);
