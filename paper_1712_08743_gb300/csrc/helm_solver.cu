@@ -486,7 +486,9 @@ static int alloc_inner(const SolveCtx& c, Inner<T>& w) {
             TRY_ALLOC(w.ph, vb, c.s); TRY_ALLOC(w.shv, vb, c.s);
         }
     }
-    return alloc_levels<T>(c.m, c.s, c.nrhs, w, c.ld > 0 ? c.ld : c.m->tail_level(sizeof(T) == 8));
+    // down to the dense level, and to the tail's first level, which takes over when an inverse could not be
+    // formed (in complex128 it lies deeper than a dense level of more than kTailMaxPoints64 nodes)
+    return alloc_levels<T>(c.m, c.s, c.nrhs, w, std::max(c.ld, c.m->tail_level(sizeof(T) == 8)));
 }
 
 // kernels one BiCGSTAB iteration launches: p, s and x/r updates plus two
@@ -932,7 +934,6 @@ static int solve_impl(const helm_model* m, cudaStream_t s, int nrhs, const doubl
             if (hs[b].outer_active) { any = 1; }
         if (!any || outer >= max_outer) break;
         if (outer == 0) {
-            // the level vectors go down to the dense level, so to the tail's first level too
             bool failed = false;
             rc = coarse_failed(*cs, s, &failed);
             if (rc == HELM_OK && failed) {
