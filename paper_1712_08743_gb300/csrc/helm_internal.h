@@ -137,7 +137,9 @@ struct DBuf {
     DBuf(const DBuf&) = delete;
     DBuf& operator=(const DBuf&) = delete;
     ~DBuf() { if (p) cudaFreeAsync(p, s); }
-    cudaError_t alloc(helm_ctx* ctx, size_t bytes, cudaStream_t st) {
+    cudaError_t alloc(helm_ctx* ctx, size_t bytes, cudaStream_t st) {   // in place of what it held
+        if (p) cudaFreeAsync(p, s);
+        p = nullptr;
         s = st;
         return pool_alloc(ctx, &p, bytes ? bytes : 16, st);
     }

@@ -786,14 +786,18 @@ static int build_coarse(const helm_model* m, cudaStream_t s, int nrhs, const dou
                                               cs.err.as<int>(), s)
                 : launch_dense_invert<float>(Ld, w2s_d, mods_d, cs.nslots, b1, b2, cs.mf.as<float>(),
                                              cs.err.as<int>(), s);
-        HELM_CUDA_TRY(e);
-        cs.slot = cs.up.at<int>(o_slot);
-        cs.grp = cs.up.at<int>(o_grp);
-        cs.ld = ld;
-        cs.n = n;
-        cs.ngroups = (int)grp.size() - 1;
-        cs.maxg = maxg;
-        return HELM_OK;
+        if (e == cudaSuccess) {
+            cs.slot = cs.up.at<int>(o_slot);
+            cs.grp = cs.up.at<int>(o_grp);
+            cs.ld = ld;
+            cs.n = n;
+            cs.ngroups = (int)grp.size() - 1;
+            cs.maxg = maxg;
+            return HELM_OK;
+        }
+        // a launch that the device refuses: the multigrid tail below takes over
+        cudaGetLastError();
+        HELM_CUDA_TRY(cudaStreamSynchronize(s));   // the host arrays are gathered anew
     }
 
     const Level& Lc = m->lv.back();
