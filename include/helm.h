@@ -151,6 +151,11 @@ const char* helm_last_error(void);
  * in the paper. */
 uint64_t helm_launch_count(void);
 
+/* Number of device allocations the library has asked for in the process so far (its
+ * contexts' pools serve them, so neither the default pool nor the free memory shows
+ * them). helm_vcycle_noalloc does not move it. */
+uint64_t helm_alloc_count(void);
+
 /* Creates a context on CUDA device `device`. `cuda_stream` (a cudaStream_t,
  * nullable) is the stream every call of this context runs on; NULL makes the
  * library create its own non-blocking stream. */

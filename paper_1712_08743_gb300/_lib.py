@@ -148,6 +148,7 @@ SIGNATURES = {
     "helm_strerror": (C.c_char_p, [_I]),
     "helm_last_error": (C.c_char_p, []),
     "helm_launch_count": (C.c_uint64, []),
+    "helm_alloc_count": (C.c_uint64, []),
     "helm_ctx_create": (_I, [_I, _P, C.POINTER(_P)]),
     "helm_ctx_destroy": (None, [_P]),
     "helm_create_model": (_I, [_P, _I, _I, _D, _pD, _I, _D, C.POINTER(_P)]),
