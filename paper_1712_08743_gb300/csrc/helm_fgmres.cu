@@ -22,6 +22,8 @@ namespace {
 constexpr int kChunk = 8;                                          // Arnoldi vectors per block in the dot products
 constexpr int kMaxChunks = (kMaxRestart - 1 + kChunk) / kChunk;     // chunks of the longest basis
 constexpr int kFgMaxBlocks = 1024;                                 // blocks per RHS (and chunk)
+constexpr int kDotThreads = 384;                                   // threads per block of the dot products
+constexpr size_t kDotMaxPts = 14;   // points that one thread adds up in FP32 when a batch's sums share a wave
 
 // Blocks per RHS of a grid-stride kernel: about two points per thread, at most
 // one wave of the kernel's resident blocks on every SM.
@@ -32,6 +34,7 @@ int fg_grid(size_t n, int share = 1) {   // share: the launch's grids (chunks, r
     static const int per_sm = [] {
         int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kernel, Threads, 0);
+        if (Threads == kDotThreads) nb = std::min(nb, 2);   // the dot products' partials in one round of loads
         return nb > 0 ? nb : 1;
     }();
     int dev = 0, sms = 0;
@@ -40,9 +43,43 @@ int fg_grid(size_t n, int share = 1) {   // share: the launch's grids (chunks, r
     const size_t cap = std::min<size_t>(kFgMaxBlocks, (size_t)std::max(1, per_sm * sms / share));
     return (int)std::max<size_t>(1, std::min<size_t>((n + 2 * Threads - 1) / (2 * Threads), cap));
 }
-constexpr int kDotThreads = 384;   // threads per block of the dot products
 // points a thread takes per step: enough loads in flight within 80 registers (two blocks per SM)
 template <typename T, int NV> constexpr int kDotPts = sizeof(T) == 8 ? (NV <= 2 ? 2 : 1) : (NV <= 4 ? 4 : NV <= 8 ? 2 : 1);
+// term(0) + .. + term(N - 1) by halves
+template <int N, typename F>
+__device__ __forceinline__ auto pairwise(F term) {
+    if constexpr (N == 4) return (term(0) + term(1)) + (term(2) + term(3));
+    else if constexpr (N == 2) return term(0) + term(1);
+    else return term(0);
+}
+// Sums of N values per lane over the warp, each in one lane: at every step half of the values go to the lane
+// `D` away and the other half is kept, so that 20 additions per lane do for 17 values where a tree for each
+// takes 85. The first two steps add in T, the others in FP64. Afterwards the lane with cnt > 0 holds the sum of
+// value `base`. Order fixed.
+template <int D, int N, typename T>
+__device__ __forceinline__ double warp_sums(const T (&v)[N], int lane, int& base, int& cnt) {
+    constexpr int H = (N + 1) / 2;
+    const bool up = lane & D;
+    T keep[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const T lo = v[i], hi = H + i < N ? v[H + i < N ? H + i : 0] : T(0);
+        keep[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, D);
+    }
+    base += up ? H : 0;
+    cnt = up ? cnt - H : min(cnt, H);
+    if constexpr (D == 1) {
+        static_assert(H == 1, "at most 32 values");
+        return (double)keep[0];
+    } else if constexpr (D == 8) {
+        double d[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) d[i] = (double)keep[i];
+        return warp_sums<D / 2>(d, lane, base, cnt);
+    } else {
+        return warp_sums<D / 2>(keep, lane, base, cnt);
+    }
+}
 }  // namespace
 
 // Partials per RHS that the FGMRES kernels need on n points: 2 kChunk + 1 sums
@@ -73,9 +110,9 @@ __global__ void k_fg_scale(const T* __restrict__ rin, T* __restrict__ v, const R
 // lane of the last block's warps takes all of its own in one round of loads, with twelve vectors
 // at a time and 1 / s_i loaded beside them. (With 256 threads: up to 912 partials, three rounds,
 // eight vectors at a time; that end was about half of a launch at one right-hand side.) On the
-// 1041 x 1041 grid: one vector 11.7 -> 9.0 us, four 13.6 -> 11.5, eight 18.3 -> 17.
+// 1041 x 1041 grid: one vector 12.4 -> 9.4 us, four 14.4 -> 12.4, eight 20 -> 16.5.
 template <typename T, int NV>
-__global__ void __launch_bounds__(kDotThreads) k_fg_dots(const T* __restrict__ V, size_t vstride, const T* __restrict__ w,
+__global__ void __launch_bounds__(kDotThreads, sizeof(T) == 8 && NV == 8 ? 1 : 2) k_fg_dots(const T* __restrict__ V, size_t vstride, const T* __restrict__ w,
                                                  int j, int add, int wnorm, int check, double* partials, int pstride,
                                                  RhsState* st, FgDev fg, size_t n) {
     constexpr int NA = 2 * NV + 1;
@@ -96,50 +133,35 @@ __global__ void __launch_bounds__(kDotThreads) k_fg_dots(const T* __restrict__ V
     T acc[NA];
 #pragma unroll
     for (int k = 0; k < NA; ++k) acc[k] = 0;
-    // kDotPts points per thread and step, every load of the step issued before use
+    // kDotPts points per thread and step, every load of the step issued before use, added by halves
     constexpr int PT = kDotPts<T, NV>;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
-    size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    for (; p + (PT - 1) * stride < n; p += PT * stride) {
+    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += PT * stride) {
         cx<T> wv[PT], q[NV][PT];
+        bool in[PT];   // the last step may be short
 #pragma unroll
-        for (int t = 0; t < PT; ++t) wv[t] = ldc(wb, p + t * stride);
+        for (int t = 0; t < PT; ++t) {
+            in[t] = t == 0 || p + t * stride < n;
+            wv[t] = in[t] ? ldc(wb, p + t * stride) : cx<T>(0, 0);
+        }
 #pragma unroll
         for (int k = 0; k < NV; ++k)
             if (k < nv)
 #pragma unroll
-                for (int t = 0; t < PT; ++t) q[k][t] = ldc(vp[k], p + t * stride);
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-            if (k < nv)
-#pragma unroll
-                for (int t = 0; t < PT; ++t) {
-                    acc[2 * k] += q[k][t].re * wv[t].re + q[k][t].im * wv[t].im;
-                    acc[2 * k + 1] += q[k][t].re * wv[t].im - q[k][t].im * wv[t].re;
-                }
-        if (wn)
-#pragma unroll
-            for (int t = 0; t < PT; ++t) acc[2 * NV] += wv[t].re * wv[t].re + wv[t].im * wv[t].im;
-    }
-    for (; p < n; p += stride) {
-        const cx<T> w0 = ldc(wb, p);
+                for (int t = 0; t < PT; ++t) q[k][t] = in[t] ? ldc(vp[k], p + t * stride) : cx<T>(0, 0);
 #pragma unroll
         for (int k = 0; k < NV; ++k)
             if (k < nv) {
-                const cx<T> q = ldc(vp[k], p);
-                acc[2 * k] += q.re * w0.re + q.im * w0.im;
-                acc[2 * k + 1] += q.re * w0.im - q.im * w0.re;
+                acc[2 * k] += pairwise<PT>([&](int t) { return q[k][t].re * wv[t].re + q[k][t].im * wv[t].im; });
+                acc[2 * k + 1] += pairwise<PT>([&](int t) { return q[k][t].re * wv[t].im - q[k][t].im * wv[t].re; });
             }
-        if (wn) acc[2 * NV] += w0.re * w0.re + w0.im * w0.im;
+        if (wn) acc[2 * NV] += pairwise<PT>([&](int t) { return wv[t].re * wv[t].re + wv[t].im * wv[t].im; });
     }
     // block reduction of the partial sums
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NA; ++k) {
-        T v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[k][warp] = (double)v;
-    }
+    int base = 0, cnt = NA;
+    const double tot = warp_sums<16>(acc, lane, base, cnt);
+    if (cnt > 0) sh[base][warp] = tot;
     __syncthreads();
     const int nblk = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
     double* part = partials + (size_t)b * pstride;
@@ -459,9 +481,18 @@ template <typename T, int NV>
 static void fg_dots_nv(const T* V, size_t vstride, const T* w, int j, int add, int wnorm, int check, double* partials,
                        int pstride, RhsState* st, const FgDev& fg, size_t n, int nrhs, cudaStream_t s) {
     const int nchunk = (j + NV) / NV;
-    // at least 16 blocks per sum: a wide batch fills the GPU by itself
+    // The sums of a launch share a wave of blocks: up to four of them as they are, more in FP32 as long as a thread has
+    // at most kDotMaxPts points or three times those of a whole wave. The rounding of its sum and of the warp's
+    // first two steps then stays at or below that of a wave of 256-thread blocks per sum whose warp tree is all
+    // in FP32 (relative rms error of two positive sums for each of 20 right-hand sides of 441 x 241: 7.6e-10 there,
+    // 6.3e-10 here, 3.0e-9 with 16 blocks per sum and such a tree; 63, 28 and 31 us).
     const int share = std::min(nchunk * nrhs, 19);
-    const dim3 grd(fg_grid<k_fg_dots<T, NV>, kDotThreads>(n, share), nchunk, nrhs);
+    int gx = fg_grid<k_fg_dots<T, NV>, kDotThreads>(n, share);
+    if (sizeof(T) == 4 && share > 4) {
+        const size_t wave = fg_grid<k_fg_dots<T, NV>, kDotThreads>(n), most = kDotMaxPts * kDotThreads;
+        gx = std::max(gx, (int)std::min((wave + 2) / 3, (n + most - 1) / most));
+    }
+    const dim3 grd(gx, nchunk, nrhs);
     // the second pass follows the first pass's update directly; the first one also waits for the
     // previous column on another stream, and is launched as an ordinary kernel
     if (add) launch_pdl(k_fg_dots<T, NV>, grd, dim3(kDotThreads), 0, s, V, vstride, w, j, add, wnorm, check, partials,

@@ -15,6 +15,7 @@ def test_noalloc_asks_for_no_memory(lib, nrhs, beta):
     import torch
 
     import paper_1712_08743_gb300 as hg
+    from paper_1712_08743_gb300.api import helm_vcycle_noalloc
 
     ctx = hg.Context(0)
     mdl = models.c1_model()
@@ -27,7 +28,7 @@ def test_noalloc_asks_for_no_memory(lib, nrhs, beta):
     assert n1 > n0
     for _ in range(2):
         z = torch.full_like(r, float("nan"))
-        hg.helm_vcycle_noalloc(model, om, r, z, beta, 0.5)
+        helm_vcycle_noalloc(model, om, r, z, beta, 0.5)
         assert lib.helm_alloc_count() == n1
         assert torch.equal(z, ref)
     model.close()
