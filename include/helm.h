@@ -398,7 +398,8 @@ int helm_vcycle_noalloc(helm_model* model, int nrhs, const double* omega, double
  * size, 32x4, 8x16, 8x8 on two threads per node, 8x16 on two threads per node), prolongation 0..4 (fine
  * tiles 16x8, by the level's size, 64x4, 32x16, 128x2);
  * the finest level's prolongation 0..1 (row segments of 16 or 32 rows); 1 is
- * the default everywhere. Batches above 16 right-hand sides have no tiles. helm_set_tiles applies a stored choice. Tile shapes
+ * the default everywhere. Batches above 16 right-hand sides have no tiles on the
+ * Galerkin levels: tuning for one leaves those choices as they are. helm_set_tiles applies a stored choice. Tile shapes
  * change the speed, not the arithmetic of a node (dot products may sum in
  * another order). */
 int helm_autotune(helm_model* model, int nrhs, double omega, int* tiles_out);

@@ -1302,6 +1302,8 @@ int autotune(helm_model* m, cudaStream_t s, int nrhs, double hw2, int reps, int*
         // the finest level's marching prolongation has two row-segment choices; the Galerkin
         // levels the tile shapes of launch_prolong_g / launch_restrict_g
         const bool fine = l == 0 && !m->vd;
+        // batches that the march takes have no tiles there: the choices of smaller batches stay
+        if (!fine && nrhs > kGalMarchMinRhs) continue;
         const int np = fine ? 2 : kProlongTiles, nr = l > 0 ? kRestrictTiles : 0;
         int bp = m->tile_prolong[l], br = m->tile_restrict[l];
         float best_p = 0.f, best_r = 0.f;
