@@ -15,6 +15,9 @@ import os
 from . import _lib
 
 NTILES = 48  # 24 levels x (restriction, prolongation)
+# What the codes mean. 6: code 1 of a Galerkin level is the rule by the level's size. Choices that were measured
+# among other shapes (stored as bare lists) are not the fastest of these, so they are measured anew.
+SHAPES = 6
 
 
 def default_cache_path() -> str:
@@ -51,12 +54,13 @@ def autotune(model, nrhs: int, omega: float, cache_path: str | None = None) -> l
     key = cache_key(model.nx, model.nz, nrhs)
     cache = load_cache(path)
     lib = model.lib
-    if key in cache and len(cache[key]) == NTILES:
-        arr = (C.c_int * NTILES)(*cache[key])
+    entry = cache.get(key)
+    if isinstance(entry, dict) and entry.get("shapes") == SHAPES and len(entry.get("tiles", ())) == NTILES:
+        arr = (C.c_int * NTILES)(*entry["tiles"])
         _lib.check(lib.helm_set_tiles(model.handle, arr), "helm_set_tiles")
-        return list(cache[key])
+        return list(entry["tiles"])
     arr = (C.c_int * NTILES)()
     _lib.check(lib.helm_autotune(model.handle, int(nrhs), float(omega), arr), "helm_autotune")
-    cache[key] = list(arr)
+    cache[key] = {"shapes": SHAPES, "tiles": list(arr)}
     save_cache(path, cache)
     return list(arr)
