@@ -523,18 +523,6 @@ static void bicg_iteration(const SolveCtx& c, Inner<T>& w) {
                       c.st, c.nactive, n, c.nrhs, c.s);
 }
 
-// Iterations in a graph, of which a whole number makes up a chunk. A node costs about 3.7 us to instantiate (ten
-// iterations of 21 kernels: 0.8 ms of a 6 ms solve), a launch about 19 us of idle GPU; for the 40 to 60 iterations of
-// a small solve the sum is least between three and five iterations, and graphs of one or two lose more
-// to their launches (82 -> 90 us per iteration with two) than longer ones to their nodes.
-int bicg_graph_iters(int chunk) {
-    for (int k = 5; k >= 3; --k)
-        if (chunk % k == 0) return k;
-    for (int k = 6; k < chunk; ++k)
-        if (chunk % k == 0) return k;
-    return chunk;
-}
-
 // Inner BiCGSTAB on rin for the right-hand sides whose outer step is active.
 // *corr: where the correction is left (w.x, or w.t when V is applied to w.x last). `graph`
 // caches the captured iteration chunk.
@@ -555,7 +543,12 @@ static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, const T** c
                             c.nrhs, c.s);
     NvtxRange nv("bicgstab inner solve");
     const int chunk = std::max(1, c.o.check_every);
-    const int per_graph = bicg_graph_iters(chunk);   // the graph is launched until the chunk is done
+    // The graph holds the largest part of a chunk up to five iterations and is launched until the
+    // chunk is done: a node costs about 3.7 us to instantiate (ten iterations of 21 kernels: 0.8 ms of
+    // a 6 ms solve), a launch about 19 us of idle GPU; for the 40 to 60 iterations of a small
+    // solve the sum is least between three and five iterations.
+    int per_graph = std::min(chunk, 5);
+    while (chunk % per_graph) --per_graph;
     if (c.o.use_graphs && *graph == nullptr) {
         cudaGraph_t g;
         HELM_CUDA_TRY(cudaStreamBeginCapture(c.s, cudaStreamCaptureModeThreadLocal));

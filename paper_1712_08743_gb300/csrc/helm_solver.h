@@ -48,8 +48,6 @@ int gn_hvp(FwiState* st, cudaStream_t s, const double* dm_dev, double* hdm_dev, 
 int gn_step(FwiState* st, cudaStream_t s, const double* g_dev, int iters, double* dm_dev, double* rel,
             const helm_solve_opts& o);
 
-int bicg_graph_iters(int chunk);   // BiCGSTAB iterations captured at a time, for a convergence check every `chunk`
-
 int coarsest_points(const helm_model* m);
 
 // One application of the multigrid preconditioner z ~ M^{-1} in (V-cycle above
