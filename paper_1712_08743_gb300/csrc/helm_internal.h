@@ -289,6 +289,7 @@ void launch_refine(const TI* x, double* u, const RhsState* st, size_t n, int nrh
 template <typename T>
 void launch_bicg_init(const T* b, T* x, T* r, T* rh, T* p, T* v, double* partials, int pstride,
                       RhsState* st, int* nactive, size_t n, int nrhs, cudaStream_t s);
+void launch_bicg_reactivate(RhsState* st, int nrhs, cudaStream_t s);
 template <typename T>
 void launch_bicg_resume(const T* rin, T* x, T* r, T* rh, T* p, T* v, double* partials, int pstride,
                         RhsState* st, int* nactive, size_t n, int nrhs, cudaStream_t s);

@@ -833,6 +833,15 @@ void launch_bicg_xr(T* x, const T* ph, const T* shv, const T* sv, const T* t, co
                sv, t, rh, r, partials, pstride, st, nactive, n);
 }
 
+// A right-hand side takes part again while its refinement goes on, whatever ended its inner solve.
+__global__ void k_bicg_reactivate(RhsState* st, int nrhs) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < nrhs) st[b].active = st[b].outer_active;
+}
+void launch_bicg_reactivate(RhsState* st, int nrhs, cudaStream_t s) {
+    k_bicg_reactivate<<<(nrhs + 127) / 128, 128, 0, s>>>(st, nrhs);
+}
+
 // ===================================================== Galerkin operators
 // Complex coefficient of stored stencil entry k (0 centre, 1 east, 2 north,
 // 3 north-east, 4 north-west) at node i: G_k - hw (b1 - j b2) K_k.

@@ -597,10 +597,10 @@ static int inner_solve(const SolveCtx& c, Inner<T>& w, const T* rin, const T** c
     }
     *corr = w.x.template as<T>();
     if (c.late_precond) {
-        SolveCtx all = c;
-        all.st = nullptr;   // every right-hand side: those that have converged are no longer active
-        vcycle<T>(all, w, w.x.template as<T>(), w.t.template as<T>(), 0, nullptr, nullptr);
-        count_launches(mg_kernels_per_apply(c.m, sizeof(T) == 8, c.lf, c.ld, c.fca ? c.fca_level : 0, c.nrhs) -
+        // for the right-hand sides of this refinement step, which are no longer active once their inner solve ended
+        launch_bicg_reactivate(c.st, c.nrhs, c.s);
+        vcycle<T>(c, w, w.x.template as<T>(), w.t.template as<T>(), 0, nullptr, nullptr);
+        count_launches(1 + mg_kernels_per_apply(c.m, sizeof(T) == 8, c.lf, c.ld, c.fca ? c.fca_level : 0, c.nrhs) -
                        (c.m->vd ? 1 : 0));
         *corr = w.t.template as<T>();
     }
