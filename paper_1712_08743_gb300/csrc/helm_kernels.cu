@@ -1419,12 +1419,12 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
 // 191 with two right-hand sides. In FP32 the skipped rows cost more in scheduling than they save (156 us).
 constexpr int PM_COLS = 60;   // fine output columns per warp
 
-template <typename T, int MODE, bool EDGE>
+template <typename T, int MODE, bool EDGE, bool OUT>
 __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, int J, int lane, int Z0, int Z1,
                                               int npml, T acoef, T hw, T b1, T b2, T wj, const T* __restrict__ fb,
                                               const T* __restrict__ eb, const T* __restrict__ ab,
                                               const T* __restrict__ m2, T* __restrict__ ob, T* __restrict__ yb,
-                                              int accumulate, bool wout, T& d0, T& d1, T& d2) {
+                                              int accumulate, T& d0, T& d1, T& d2) {
     const int c0 = 2 * J;
     const bool in0 = !EDGE || (c0 >= 0 && c0 < nx), in1 = !EDGE || (c0 + 1 >= 0 && c0 + 1 < nx);
     const bool ein = !EDGE || (J >= 0 && J < cnx);
@@ -1559,7 +1559,7 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
                 if (h) arow(z, RB, qb0, qb1, qc0, qc1, qd0, qd1, y0, y1);
                 else arow(z, RA, qa0, qa1, qb0, qb1, qc0, qc1, y0, y1);
                 if (wr) {
-                    if (MODE == 3 || wout) {
+                    if constexpr (OUT) {
                         if (in0) stc(ob, i, c0v);
                         if (in1) stc(ob, i + 1, c1v);
                     }
@@ -1591,7 +1591,9 @@ __device__ __forceinline__ void prolong_march(int nx, int nz, int cnx, int cnz, 
 
 constexpr int PM_WARPS = 4;   // most warps per block of the marching prolongation
 
-template <typename T, int MODE>
+// OUT: modes 1 to 3 write the cycle's result too, not only A times it. A template parameter: as a test of the pointer
+// it cost the launches that write 6 % (ten right-hand sides of 1041 x 1041: 96.5 -> 103.7 us).
+template <typename T, int MODE, bool OUT = true>
 __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev Lc, int npml, T acoef,
                                                  const T* __restrict__ w2, T b1, T b2, T wj,
                                                  const T* __restrict__ f, const T* __restrict__ ec,
@@ -1622,11 +1624,11 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_prolong(LevelDev Lf, LevelDev
         const bool edge = Jb < 0 || 2 * Jb + 63 >= nx || Jb + 31 >= cnx || Z0 < 4 || Z1 + 3 >= nz ||
                           Z0 / 2 - 2 < 0 || Z1 / 2 + 2 >= cnz;
         if (edge)
-            prolong_march<T, MODE, true>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
-                                         eb, ab, m2, ob, yb, accumulate, out != nullptr, d0, d1, d2);
+            prolong_march<T, MODE, true, OUT>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
+                                         eb, ab, m2, ob, yb, accumulate, d0, d1, d2);
         else
-            prolong_march<T, MODE, false>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
-                                          eb, ab, m2, ob, yb, accumulate, out != nullptr, d0, d1, d2);
+            prolong_march<T, MODE, false, OUT>(nx, nz, cnx, cnz, Jb + lane, lane, Z0, Z1, npml, acoef, hw, b1, b2, wj, fb,
+                                          eb, ab, m2, ob, yb, accumulate, d0, d1, d2);
     }
     if constexpr (MODE == 0 || MODE == 3) return;
     else {
@@ -1693,11 +1695,11 @@ void launch_prolong(int mode, const LevelDev& Lf, const LevelDev& Lc, int npml, 
         launch_pdl(k_prolong<T, 0>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
     else if (mode == 1)
-        launch_pdl(k_prolong<T, 1>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
-                   partials, pstride, st, accumulate, zs);
+        launch_pdl(out ? k_prolong<T, 1> : k_prolong<T, 1, false>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2,
+                   (T)wj, f, ec, out, y, aux, partials, pstride, st, accumulate, zs);
     else if (mode == 2)
-        launch_pdl(k_prolong<T, 2>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
-                   partials, pstride, st, accumulate, zs);
+        launch_pdl(out ? k_prolong<T, 2> : k_prolong<T, 2, false>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2,
+                   (T)wj, f, ec, out, y, aux, partials, pstride, st, accumulate, zs);
     else
         launch_pdl(k_prolong<T, 3>, grd, dim3(block), 0, s, Lf, Lc, npml, ac, w2, (T)b1, (T)b2, (T)wj, f, ec, out, y, aux,
                    partials, pstride, st, accumulate, zs);
