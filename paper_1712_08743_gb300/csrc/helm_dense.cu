@@ -53,7 +53,7 @@ __device__ __forceinline__ double2 gal_raw(const double* __restrict__ gk, size_t
 // for i < j; G_ji = G_ij^T. That is n^2 w operations in place of n^3, and its serial
 // part is n pivots of a w x w matrix held in one block's registers (one block barrier
 // each), in place of n / 8 strip steps with a grid barrier each. On the 1024-node
-// level of a 1041 x 1041 grid (complex64) the three launches take 226 us where a strip
+// level of a 1041 x 1041 grid (complex64) the three launches take 242 us where a strip
 // elimination of the whole matrix took 2843 us; on 690 nodes in complex128, bound by the
 // FP64 rate and latency of the two SMs that run the chains, 2.0 ms instead of 8.2 ms. Its
 // error in complex64 is that of the strip elimination (2-norm, five levels of 441 to 1024

@@ -1413,7 +1413,8 @@ void launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* w2, double
 // rows ahead; neighbours across a lane boundary come by shuffle.
 // FP32 on 320 right-hand sides of 441 x 241: 16 warps per SM (registers) that issue in 50 to 70 % of
 // the cycles, waiting for loads otherwise. The damping terms only where a row or the warp's columns have
-// any, and packed sums: 142 -> 128 us. A cap of 128 registers for mode 1 spills (137 us). FP64 is bound
+// any, and packed sums: 142 -> 128 us, 118 us with OUT as a template parameter. A cap of 128 registers for mode 1
+// spills (137 us). FP64 is bound
 // by its arithmetic at two results per clock and SM: the first step's unused u3, the rows above
 // the segment and the second divide of odd rows left out, blocks without idle warps: 80 -> 39 us on 241 x
 // 191 with two right-hand sides. In FP32 the skipped rows cost more in scheduling than they save (156 us).
