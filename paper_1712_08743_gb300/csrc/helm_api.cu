@@ -88,6 +88,7 @@ int create_model(helm_ctx* ctx, cudaStream_t s, int Px, int Pz, double h, const 
     DeviceGuard g(ctx->device);
     helm_model* m = new helm_model();
     m->ctx = ctx;
+    m->device = ctx->device;
     m->Px = Px; m->Pz = Pz; m->npml = npml; m->h = h; m->alpha_max = alpha_max;
     m->nx = Px + 2 * npml; m->nz = Pz + 2 * npml;
     m->nmodels = nmodels;
@@ -296,7 +297,7 @@ int helm_create_model_rho(helm_ctx* ctx, int Px, int Pz, double h, const double*
 
 void helm_destroy_model(helm_model* m) {
     if (!m) return;
-    DeviceGuard g(m->ctx->device);
+    DeviceGuard g(m->device);
     if (m->slab) cudaFree(m->slab);   // no call leaves work on it behind (Drain); the memory returns to the context's pool
     delete m;
 }

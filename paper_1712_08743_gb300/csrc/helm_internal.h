@@ -90,6 +90,7 @@ struct helm_ctx {
 };
 
 struct helm_model {
+    int device = 0;                       // the context's, for a model that is destroyed after it
     helm_ctx* ctx = nullptr;
     int Px = 0, Pz = 0, npml = 0, nx = 0, nz = 0;
     double h = 0, alpha_max = 0;
